@@ -118,11 +118,11 @@ __device__ void visit_tile_coop(const EngineArgs &a, const ImageView &im, uint32
     // its current halo
     bool settled = false;
     for (;;) {
-        uint32_t rows = 0;
+        uint32_t rows = RT::template absorb_side<IWPP_CHG_XOR>(hx, J, I);
         bool up_fresh = false;   // the strip's last pass was an up pass run with its current halo
         for (;;) {   // joint iterations of the strips
             if (!settled) {
-                const uint32_t chd = RT::template pass_down<IWPP_CHG_XOR>(hx, J, I, jt, lane);
+                const uint32_t chd = RT::template pass_down<IWPP_CHG_XOR>(J, I, jt);
                 passes++;
                 rows |= chd;
                 // A down pass that changes nothing right after an up pass with the same halo
@@ -131,7 +131,7 @@ __device__ void visit_tile_coop(const EngineArgs &a, const ImageView &im, uint32
                 if (up_fresh && !__any_sync(0xffffffffu, chd != 0)) {
                     settled = true;
                 } else {
-                    const uint32_t chu = RT::template pass_up<IWPP_CHG_XOR>(hx, J, I, jb, lane);
+                    const uint32_t chu = RT::template pass_up<IWPP_CHG_XOR>(J, I, jb);
                     passes++;
                     rows |= chu;
                     // likewise an up pass that changes nothing after a down pass with the same
@@ -344,7 +344,7 @@ __device__ void scan_tile_coop(const EngineArgs &a, const ImageView &im, uint32_
 // 16-row strip of a tile with its halo, checks the precondition and whether one of its
 // pixels can rise; a strip that can makes its tile PENDING (batches: a fire-and-forget OR)
 // or notifies it (single images: the first notification queues the tile, later ones find it
-// PENDING). Warps go from strip to strip independently, 7 CTAs per SM. The streaming scan
+// PENDING). Warps go from strip to strip independently, 7 CTAs per SM. The block scan
 // (iwpp_scan.cuh) replaces it wherever one connectivity is compiled in; the mixed-kind build
 // keeps it (its kinds switch per strip).
 #ifndef IWPP_SCAN_STRIP_MINB

@@ -32,6 +32,7 @@ __device__ __forceinline__ uint32_t min2(uint32_t a, uint32_t b) {
     asm("min.u16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
     return d;
 }
+__device__ __forceinline__ uint32_t max3(uint32_t a, uint32_t b, uint32_t c) { return __vimax3_u16x2(a, b, c); }
 // Left neighbours of a packed pair: (column 2c - 1, column 2c) from the previous lane's
 // pair `p` and this lane's pair `v`; right neighbours: (column 2c + 1, column 2c + 2).
 __device__ __forceinline__ uint32_t left_of(uint32_t p, uint32_t v) { return __byte_perm(p, v, 0x5432); }
@@ -330,47 +331,74 @@ struct RegTile {
         return lane == 0 ? s.hxJ : (lane == 31 ? s.hxJ + TH + 2 : s.hzero);
     }
 
+    // Horizontal max of a packed row over (left, self, right) inside the tile: lane 0's up shuffle
+    // and lane 31's down shuffle return their own pair, whose outside neighbour then repeats a pixel
+    // of the pair.
+    static __device__ __forceinline__ uint32_t hmax_in(uint32_t v) {
+        const uint32_t p = __shfl_up_sync(0xffffffffu, v, 1), n = __shfl_down_sync(0xffffffffu, v, 1);
+        return max3(v, left_of(p, v), right_of(v, n));
+    }
+
+    // Raise the side columns' pixels by what the side halo offers them: J <- min(I, max(J, halo
+    // pixels beside it)). The halo is fixed while the tile is being settled, so doing it once
+    // leaves the side halo out of every row step of the passes. Returns as the passes do.
+    template <bool DIFF = false>
+    static __device__ __forceinline__ uint32_t absorb_side(const uint32_t *hx, uint32_t (&J)[TH],
+                                                           const uint32_t (&I)[TH]) {
+        uint32_t chg = 0, h0 = hx[0], h1 = hx[1];
+#pragma unroll
+        for (int r = 0; r < TH; r++) {
+            const uint32_t h2 = CONN == 8 || r + 2 <= TH ? hx[r + 2] : 0u;
+            const uint32_t nv = min2(I[r], CONN == 8 ? max2(J[r], max3(h0, h1, h2)) : max2(J[r], h1));
+            if (DIFF) chg |= nv ^ J[r];
+            else chg |= (uint32_t)(nv != J[r]) << r;
+            J[r] = nv;
+            h0 = h1;
+            h1 = h2;
+        }
+        return chg;
+    }
+
     // One down pass; returns this lane's mask of changed rows. For 8-connectivity the
     // neighbourhood {W, E, N, NW, NE} of a row is the horizontal max of max(row, row above)
-    // (max commutes with the shift), so one shuffle pair per row serves both rows; the
-    // side halo is then the max of the two rows' halo words. For 4-connectivity each row
-    // first takes N (clamped to I: a valid update of every pixel) and then W / E from
-    // those new values, so a path that steps down and sideways advances within one pass
-    // (measured: 7 instead of 16 passes per visit on the 4096^2 tissue image).
+    // (max commutes with the shift), so one shuffle pair per row serves both rows. For
+    // 4-connectivity each row first takes N (clamped to I: a valid update of every pixel) and then
+    // W / E from those new values, so a path that steps down and sideways advances within one pass
+    // (measured: 7 instead of 16 passes per visit on the 4096^2 tissue image). The side halo has
+    // been absorbed before (absorb_side): a row step is 6 arithmetic instructions (with
+    // 3-input maxima; 9 and a shared load when each step took the side halo in). They bound the
+    // drain: min/max.u16x2 and byte permutes issue every second cycle of a scheduler, shuffles every
+    // fourth (measured).
     // DIFF: return the OR of (new ^ old) over the rows instead of the mask of changed rows
     // (non-zero iff this lane changed a pixel; one instruction per row instead of three).
     template <bool DIFF = false>
-    static __device__ __forceinline__ uint32_t pass_down(const uint32_t *hx, uint32_t (&J)[TH],
-                                                         const uint32_t (&I)[TH], uint32_t jt, int lane) {
-        uint32_t chg = 0, up = jt, hprev = hx[0];
+    static __device__ __forceinline__ uint32_t pass_down(uint32_t (&J)[TH], const uint32_t (&I)[TH], uint32_t jt) {
+        uint32_t chg = 0, up = jt;
 #pragma unroll
         for (int r = 0; r < TH; r++) {
-            const uint32_t hcur = hx[r + 1], v = J[r];
-            const uint32_t nv = CONN == 8 ? min2(I[r], hmax(max2(v, up), max2(hcur, hprev), lane))
-                                          : min2(I[r], hmax(min2(I[r], max2(v, up)), hcur, lane));
+            const uint32_t v = J[r];
+            const uint32_t nv = CONN == 8 ? min2(I[r], hmax_in(max2(v, up)))
+                                          : min2(I[r], hmax_in(min2(I[r], max2(v, up))));
             if (DIFF) chg |= nv ^ v;
             else chg |= (uint32_t)(nv != v) << r;
             J[r] = nv;
             up = nv;
-            hprev = hcur;
         }
         return chg;
     }
 
     template <bool DIFF = false>
-    static __device__ __forceinline__ uint32_t pass_up(const uint32_t *hx, uint32_t (&J)[TH],
-                                                       const uint32_t (&I)[TH], uint32_t jb, int lane) {
-        uint32_t chg = 0, dn = jb, hnext = hx[TH + 1];
+    static __device__ __forceinline__ uint32_t pass_up(uint32_t (&J)[TH], const uint32_t (&I)[TH], uint32_t jb) {
+        uint32_t chg = 0, dn = jb;
 #pragma unroll
         for (int r = TH - 1; r >= 0; r--) {
-            const uint32_t hcur = hx[r + 1], v = J[r];
-            const uint32_t nv = CONN == 8 ? min2(I[r], hmax(max2(v, dn), max2(hcur, hnext), lane))
-                                          : min2(I[r], hmax(min2(I[r], max2(v, dn)), hcur, lane));
+            const uint32_t v = J[r];
+            const uint32_t nv = CONN == 8 ? min2(I[r], hmax_in(max2(v, dn)))
+                                          : min2(I[r], hmax_in(min2(I[r], max2(v, dn))));
             if (DIFF) chg |= nv ^ v;
             else chg |= (uint32_t)(nv != v) << r;
             J[r] = nv;
             dn = nv;
-            hnext = hcur;
         }
         return chg;
     }
@@ -712,14 +740,14 @@ __device__ void visit_tile_reg(const EngineArgs &a, const ImageView &im, uint32_
     IWPP_RT_MARK(0);
     uint32_t passes = 0;
     for (;;) {
-        uint32_t rows = 0;
+        uint32_t rows = RT::absorb_side(hx, J, I);
         for (;;) {
 #if IWPP_REG_SWEEPS
             uint32_t ch = RT::sweep_raster(hx, J, I, jt, lane);
             ch |= RT::sweep_antiraster(hx, J, I, jb, lane);
 #else
-            uint32_t ch = RT::pass_down(hx, J, I, jt, lane);
-            ch |= RT::pass_up(hx, J, I, jb, lane);
+            uint32_t ch = RT::pass_down(J, I, jt);
+            ch |= RT::pass_up(J, I, jb);
 #endif
             passes += 2;
             rows |= ch;
