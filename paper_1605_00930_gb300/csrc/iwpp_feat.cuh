@@ -1,8 +1,8 @@
 // iwpp_feat.cuh — the learned work estimator's per-block features (include/iwpp.h): the
 // per-pixel accumulation and the conversion of a block's exact integer sums to the 16 FP32
 // inputs of the MLP. Shared by the stand-alone features kernel (iwpp_sched.cu) and the
-// streaming scan kernel, which computes the features of the tile it streams through
-// (iwpp_scan.cuh), so that both give identical values.
+// block scan kernel, which computes the features of the tile it tests (iwpp_scan.cuh), so
+// that both give identical values.
 //
 // Per 64 x 64 block, in the dilation domain (erosion: both images complemented), with
 // d = max(I - J, 0) and d8 = d (u8) or d >> 8 (u16); f[0..14] over every kFeatRowStep-th row

@@ -1,18 +1,23 @@
-// iwpp_scan.cuh — the streaming scan of the cooperative solver's 64 x 64 tiles (sm_103a).
+// iwpp_scan.cuh — the scan of the cooperative solver's 64 x 64 tiles (sm_103a).
 //
 // The scan is the initialisation pass of Algorithm 7 reduced to what the persistent drain
 // needs: per tile, whether the precondition J <= I holds and whether one step of the update
 // (Eq. "recon") would raise one of its pixels, in which case the tile enters the queue. It
 // reads every pixel once, so it is bound by HBM and by how many loads are in flight.
 //
-// One warp streams one tile from the halo row above it to the halo row below it; lane c
-// holds columns 2c and 2c + 1 of a row (u16x2, dilation domain), lanes 0 and 31 also the
-// halo column pixel on their side. Loads run IWPP_STREAM_DEPTH rows ahead of the row
-// being tested, through a ring of registers, so every warp keeps that many rows in flight without
-// a break between tiles, and the image table is read once per tile. Rows are tested with a
-// sliding window of three rows; learned batches also add up the tile's feature sums over its
-// sampled rows (iwpp_feat.cuh) and, as the warp owns the whole tile, write its 16 features
-// directly.
+// One warp tests a strip of 16 rows x 64 columns at a time (a tile is four strips) as a 4 x 8
+// grid of lane blocks: lane (lr, lc) = (lane / 8, lane % 8) holds rows 4 lr .. + 3 and columns
+// 8 lc .. + 7, with the row above and below them. Rows are read in 8-pixel spans, one 64-bit
+// (u8) or 128-bit (u16) load where the image's width keeps spans aligned, else 32-bit words
+// joined by funnel shifts, and every load of the strip is issued before the first is used:
+// one memory round trip per strip, 2-4 KB in flight per warp. (A scan that streamed a tile row
+// by row through one warp, 2 pixels per lane and two rows ahead, took 33 round trips per tile:
+// 512^2 u8 34 us against 8 now, 4096^2 u8 40 against 18, 16384^2 u8 482 against 195 (2.8 TB/s),
+// 48 u8 + u16 images of 166 MB 245 against 153, 256 images with features 1.43 ms against 1.08.)
+// Word k (k = 0..3) of a row packs the block's columns k and k + 4 as u16x2 in the dilation domain, so that horizontal
+// neighbours are other words of the lane but for the block's edges (two shuffles per row). Learned batches
+// also add up the tile's feature sums over its sampled rows (iwpp_feat.cuh): there a warp
+// takes the tile's four strips in turn and writes its 16 features.
 #pragma once
 #include <type_traits>
 
@@ -21,179 +26,256 @@
 
 namespace iwpp {
 
-#ifndef IWPP_STREAM_DEPTH
-#define IWPP_STREAM_DEPTH 2   // rows of loads in flight per warp (4, 6, 8: slower, measured)
+// CTAs (of 4 warps) per SM: one pixel type 8 (64 registers; 12 and 6 are slower, 4096^2 u8 18.1 us
+// against 24.3 and 19.7), u8 + u16 6 (their variants spill at 64: 48 images 153 us against 161),
+// with the feature sums 4 (256 images: 1.08 ms against 1.20 with 6 and 1.27 with 5).
+#ifndef IWPP_SCAN_MINB
+#define IWPP_SCAN_MINB 8
 #endif
-#ifndef IWPP_STREAM_MINB
-#define IWPP_STREAM_MINB 8    // CTAs (of 4 warps) per SM of the streaming scan
+#ifndef IWPP_SCAN_ANY_MINB
+#define IWPP_SCAN_ANY_MINB 6
 #endif
-#ifndef IWPP_STREAM_FEATS_MINB
-#define IWPP_STREAM_FEATS_MINB 8   // the same with the feature sums (spills, but faster than 6 or 7: measured)
+#ifndef IWPP_SCAN_FEATS_MINB
+#define IWPP_SCAN_FEATS_MINB 4
 #endif
 
-// One row of the stream as loaded; unpacked only when the row is used, so that the loads of
-// the rows ahead stay in flight.
-struct StreamRow {
-    uint32_t j0, j1, i0, i1, h;
-};
+constexpr int kScanRows = 4;   // rows per lane block
 
-// Loads of image row y (clamped into the image, so every address is valid; rows and columns
-// outside it are zeroed by stream_unpack). PAIR: W even, so the pair (gx, gx + 1) is one
-// aligned two-element load; else two element loads. Lanes 0 and 31 load their halo column
-// pixel `hc`. needI: the mask row is used (not for the halo rows above and below the tile).
-template <bool WIDE, bool PAIR>
-__device__ __forceinline__ void stream_issue(const ImageView &im, int y, int gx, int hc, bool needI, int lane,
-                                             StreamRow &r) {
-    using E = typename std::conditional<WIDE, uint16_t, uint8_t>::type;
-    const E *J = reinterpret_cast<const E *>(im.J);
-    const E *I = reinterpret_cast<const E *>(im.I);
+// How an image's rows can be read at a strip: aligned 8-pixel spans (width a multiple of 8),
+// or aligned 32-bit words (every other width of 8 or more). Images narrower than 8 pixels, and
+// strips that reach (with their halo row) the image's last pixels when those do not fill a
+// word, go pixel by pixel, so that nothing outside the buffers is touched.
+enum ScanMode { kScanSpan, kScanWord, kScanPixel };
+__device__ __forceinline__ ScanMode scan_mode(const ImageView &im, bool w16, int y0, int x0) {
+    if ((im.W & 7) == 0) return kScanSpan;
+    const bool last = y0 + kCoopStrip + 1 >= im.H && x0 + 64 + 3 >= im.W;
+    const bool tail = (((((uint32_t)im.H & 3u) * ((uint32_t)im.W & 3u)) << (w16 ? 1 : 0)) & 3u) != 0;
+    return im.W < 8 || (last && tail) ? kScanPixel : kScanWord;
+}
+
+// The raw words of pixels (y, x .. x + 7) at clamped addresses (what lies outside the image is
+// masked by the caller): span u8 2 / u16 4 words; word u8 3 / u16 5, joined by scan_join.
+template <bool W16, int M>
+__device__ __forceinline__ void scan_issue(const ImageView &im, const uint8_t *p, int y, int x, uint32_t (&v)[5]) {
     const size_t row = (size_t)min(max(y, 0), im.H - 1) * (size_t)im.W;
-    if (PAIR) {
-        using P = typename std::conditional<WIDE, uint32_t, uint16_t>::type;
-        const size_t e = row + (size_t)min(gx, im.W - 2);
-        r.j0 = __ldg(reinterpret_cast<const P *>(J + e));
-        r.i0 = needI ? (uint32_t)__ldg(reinterpret_cast<const P *>(I + e)) : 0u;
-    } else {
-        const size_t e0 = row + (size_t)min(gx, im.W - 1), e1 = row + (size_t)min(gx + 1, im.W - 1);
-        r.j0 = __ldg(J + e0);
-        r.j1 = __ldg(J + e1);
-        r.i0 = needI ? (uint32_t)__ldg(I + e0) : 0u;
-        r.i1 = needI ? (uint32_t)__ldg(I + e1) : 0u;
-    }
-    r.h = (lane == 0 || lane == 31) ? (uint32_t)__ldg(J + row + (size_t)min(max(hc, 0), im.W - 1)) : 0u;
-}
-
-// The row in the dilation domain: packed pair of J and I (0 outside the image) and this
-// lane's halo word (lane 0: left halo pixel, lane 31: right halo pixel << 16, as hmax wants).
-template <bool WIDE, bool PAIR>
-__device__ __forceinline__ void stream_unpack(const StreamRow &r, bool yin, uint32_t cm, uint32_t flip, bool hin,
-                                              int lane, uint32_t &J, uint32_t &I, uint32_t &H) {
-    uint32_t j, i;
-    if (PAIR) {
-        j = WIDE ? r.j0 : __byte_perm(r.j0, 0u, 0x4140);
-        i = WIDE ? r.i0 : __byte_perm(r.i0, 0u, 0x4140);
-    } else {
-        j = r.j0 | (r.j1 << 16);
-        i = r.i0 | (r.i1 << 16);
-    }
-    const uint32_t f2 = flip | (flip << 16);
-    J = yin ? (j ^ f2) & cm : 0u;
-    I = yin ? (i ^ f2) & cm : 0u;
-    H = (yin && hin) ? (r.h ^ flip) << (lane == 31 ? 16 : 0) : 0u;
-}
-
-// One tile: rows y0 .. y0 + ny - 1 of the image (ny >= 1), streamed as rows y0 - 1 .. y0 + ny.
-// Sets `can` (a pixel can rise: min(I, max over its neighbourhood of J) != J) and `bad`
-// (J > I somewhere) for this lane; FEATS: adds the tile's pixels to `fa`.
-template <bool WIDE, bool PAIR, int CONN, bool FEATS>
-__device__ __forceinline__ void scan_tile_stream(const ImageView &im, int y0, int x0, int ny, int lane,
-                                                 bool &can, bool &bad, FeatAcc &fa) {
-    using RT = RegTile<uint8_t, CONN, kCoopStrip>;   // hmax only (independent of the pixel type)
-    constexpr int D = IWPP_STREAM_DEPTH;
-    const int gx = x0 + 2 * lane;
-    const int hc = lane == 0 ? x0 - 1 : x0 + RT::TW;
-    const bool hin = (lane == 0 && x0 > 0) || (lane == 31 && x0 + RT::TW < im.W);
-    const bool c0 = gx < im.W, c1 = gx + 1 < im.W;
-    const uint32_t cm = (c0 ? 0xFFFFu : 0u) | (c1 ? 0xFFFF0000u : 0u);
-    const uint32_t rm = (c1 ? 0xFFFFu : 0u) | (lane < 31 && gx + 2 < im.W ? 0xFFFF0000u : 0u);   // right neighbour counts
-    const uint32_t thr = 16u * ((WIDE ? 0xFFFFu : 0xFFu) / 255u);
-    const int ns = ny + 2;   // stream rows: s <-> image row y0 - 1 + s
-    StreamRow q[D];
+    if (M == kScanSpan) {
+        const size_t e = row + (size_t)min(x, im.W - 8);
+        if (W16) {
+            const uint4 u = __ldg(reinterpret_cast<const uint4 *>(p + 2 * e));
+            v[0] = u.x; v[1] = u.y; v[2] = u.z; v[3] = u.w;
+        } else {
+            const uint2 u = __ldg(reinterpret_cast<const uint2 *>(p + e));
+            v[0] = u.x; v[1] = u.y;
+        }
+    } else if (M == kScanWord) {
+        const size_t a = (row + (size_t)min(x, im.W - 1)) << (W16 ? 1 : 0), a4 = a & ~(size_t)3;
+        const size_t last = ((((size_t)im.H * (size_t)im.W) << (W16 ? 1 : 0)) - 4) & ~(size_t)3;   // last whole word
 #pragma unroll
-    for (int k = 0; k < D; k++)
-        if (k < ns) stream_issue<WIDE, PAIR>(im, y0 - 1 + k, gx, hc, k >= 1 && k <= ny, lane, q[k]);
-    uint32_t jPrev = 0, jCur = 0, iCur = 0, hPrev = 0, hCur = 0;
-    uint32_t h03 = 0, h47 = 0;   // FEATS: 8-bit histogram bins (at most 32 sampled pixels per lane)
-    bool any = false, nok = false;
-    for (int s0 = 0; s0 < ns; s0 += D) {
-#pragma unroll
-        for (int k = 0; k < D; k++) {
-            const int s = s0 + k;
-            if (s < ns) {   // warp-uniform
-                const int y = y0 - 1 + s;
-                uint32_t Jn, In, Hn;
-                stream_unpack<WIDE, PAIR>(q[k], y >= 0 && y < im.H, cm, im.flip, hin, lane, Jn, In, Hn);
-                if (s + D < ns) stream_issue<WIDE, PAIR>(im, y + D, gx, hc, s + D <= ny, lane, q[k]);
-                const uint32_t hN = RT::hmax(Jn, Hn, lane);
-                if (s >= 2) {   // test row s - 1 of the stream (a row of the tile)
-                    const uint32_t m = CONN == 8 ? max2(hPrev, max2(hCur, hN)) : max2(hCur, max2(jPrev, Jn));
-                    any |= min2(iCur, m) != jCur;
-                    nok |= max2(jCur, iCur) != iCur;
-                    if (FEATS && ((s - 2) % kFeatRowStep) == 0) {   // a sampled row (tile row s - 2)
-                        const uint32_t iv = iCur, jv = jCur;
-                        const uint32_t dv = max2(iv, jv) - jv;   // per half max(I - J, 0): no borrow
-                        const uint32_t d8 = WIDE ? (dv >> 8) & 0x00FF00FFu : dv;
-                        const uint32_t bl = min(7u, 32u - (uint32_t)__clz(d8 & 0xFFFFu));   // bit length, 0 for 0
-                        const uint32_t bh = min(7u, 32u - (uint32_t)__clz(d8 >> 16));
-                        h03 += (bl < 4 ? 1u << (8 * bl) : 0u) + (bh < 4 ? 1u << (8 * bh) : 0u);
-                        h47 += (bl >= 4 ? 1u << (8 * bl - 32) : 0u) + (bh >= 4 ? 1u << (8 * bh - 32) : 0u);
-                        const uint32_t x = iv ^ jv;
-                        fa.seeds += (uint32_t)((x & 0xFFFFu) == 0 && (jv & 0xFFFFu) != 0) +
-                                    (uint32_t)((x >> 16) == 0 && (jv >> 16) != 0);
-                        fa.sI = __dp2a_lo(iv, 0x0101u, fa.sI);
-                        fa.sJ = __dp2a_lo(jv, 0x0101u, fa.sJ);
-                        fa.sD = __dp2a_lo(dv, 0x0101u, fa.sD);
-                        fa.sI2 += (unsigned long long)(iv & 0xFFFFu) * (iv & 0xFFFFu);
-                        fa.sI2 += (unsigned long long)(iv >> 16) * (iv >> 16);
-                        fa.sJ2 += (unsigned long long)(jv & 0xFFFFu) * (jv & 0xFFFFu);
-                        fa.sJ2 += (unsigned long long)(jv >> 16) * (jv >> 16);
-                        // edges: the right neighbours in the tile, the pixel below in the tile
-                        const uint32_t rp = __byte_perm(iv, __shfl_down_sync(0xffffffffu, iv, 1), 0x5432);
-                        const uint32_t gxv = (max2(iv, rp) - min2(iv, rp)) & rm;
-                        const uint32_t gyv = s <= ny ? max2(iv, In) - min2(iv, In) : 0u;
-                        fa.edges += (uint32_t)((gxv & 0xFFFFu) + (gyv & 0xFFFFu) > thr) +
-                                    (uint32_t)((gxv >> 16) + (gyv >> 16) > thr);
-                    }
-                }
-                jPrev = jCur;
-                jCur = Jn;
-                iCur = In;
-                hPrev = hCur;
-                hCur = hN;
-            }
+        for (int i = 0; i < (W16 ? 5 : 3); i++) {
+            const size_t o = a4 + 4 * i;
+            v[i] = __ldg(reinterpret_cast<const uint32_t *>(p + (o < last ? o : last)));
+        }
+    } else {
+        v[0] = v[1] = v[2] = v[3] = 0;
+        for (int k = 0; k < 8; k++) {
+            const size_t e = row + (size_t)min(x + k, im.W - 1);
+            const uint32_t q = W16 ? (uint32_t)__ldg(reinterpret_cast<const uint16_t *>(p) + e) : (uint32_t)__ldg(p + e);
+            const uint32_t s = q << (W16 ? 16 * (k & 1) : 8 * (k & 3));
+            const int d = W16 ? k >> 1 : k >> 2;
+            v[0] |= d == 0 ? s : 0u;
+            v[1] |= d == 1 ? s : 0u;
+            v[2] |= d == 2 ? s : 0u;
+            v[3] |= d == 3 ? s : 0u;
         }
     }
-    can = any;
-    bad = nok;
-    if (FEATS) {
-        const uint32_t nrs = (uint32_t)((ny + kFeatRowStep - 1) / kFeatRowStep);   // sampled rows
-        fa.n = nrs * ((uint32_t)c0 + (uint32_t)c1);
-        fa.npix = (uint32_t)ny * ((uint32_t)c0 + (uint32_t)c1);
-        fa.h03 = h03 - (2u * nrs - fa.n);   // columns outside the image were counted in bin 0
-        fa.h47 = h47;
+}
+// The issued words as words (k, k + 4) in the dilation domain, 0 outside the image.
+template <bool W16, int M>
+__device__ __forceinline__ void scan_unpack(const ImageView &im, int y, int x, const uint32_t (&cm)[4],
+                                            const uint32_t (&t)[5], uint32_t (&o)[4]) {
+    uint32_t v[4] = {t[0], t[1], t[2], t[3]};
+    if (M == kScanWord) {
+        const size_t a = ((size_t)min(max(y, 0), im.H - 1) * (size_t)im.W + (size_t)min(x, im.W - 1)) << (W16 ? 1 : 0);
+        const uint32_t sh = 8u * (uint32_t)(a & 3);
+#pragma unroll
+        for (int i = 0; i < (W16 ? 4 : 2); i++) v[i] = __funnelshift_r(t[i], t[i + 1], sh);
+    }
+    if (W16) {
+        o[0] = __byte_perm(v[0], v[2], 0x5410);
+        o[1] = __byte_perm(v[0], v[2], 0x7632);
+        o[2] = __byte_perm(v[1], v[3], 0x5410);
+        o[3] = __byte_perm(v[1], v[3], 0x7632);
+    } else {
+        const uint32_t a = __byte_perm(v[0], v[1], 0x5410), b = __byte_perm(v[0], v[1], 0x7632);
+        o[0] = __byte_perm(a, 0u, 0x4240);
+        o[1] = __byte_perm(a, 0u, 0x4341);
+        o[2] = __byte_perm(b, 0u, 0x4240);
+        o[3] = __byte_perm(b, 0u, 0x4341);
+    }
+    const uint32_t f2 = im.flip | (im.flip << 16);
+    const bool in = y >= 0 && y < im.H;
+#pragma unroll
+    for (int k = 0; k < 4; k++) o[k] = in ? (o[k] ^ f2) & cm[k] : 0u;
+}
+
+// One strip: rows y0 .. y0 + 15 (y0 < H), columns x0 .. x0 + 63. Sets `can` (a pixel can rise:
+// min(I, max over its neighbourhood of J) != J) and `bad` (J > I somewhere) for this lane; FEATS:
+// adds the lane's pixels to `fa`.
+template <bool W16, int M, int CONN, bool FEATS>
+__device__ __forceinline__ void scan_strip(const ImageView &im, int y0, int x0, int lane, bool &can, bool &bad,
+                                           FeatAcc &fa) {
+    constexpr int RB = kScanRows;
+    const int lr = lane >> 3, lc = lane & 7;
+    const int y = y0 + RB * lr, x = x0 + 8 * lc;
+    uint32_t rj[RB + 2][5], ri[RB][5];
+#pragma unroll
+    for (int r = 0; r < RB + 2; r++) scan_issue<W16, M>(im, im.J, y + r - 1, x, rj[r]);
+#pragma unroll
+    for (int r = 0; r < RB; r++) scan_issue<W16, M>(im, im.I, y + r, x, ri[r]);
+    // side halo: lanes lc == 0 read column x0 - 1, lanes lc == 7 column x0 + 64
+    const int xs = lc == 0 ? x0 - 1 : x0 + 64;
+    const bool xin = (lc == 0 && xs >= 0) || (lc == 7 && xs < im.W);
+    uint32_t hs[RB + 2];
+#pragma unroll
+    for (int r = 0; r < RB + 2; r++) {
+        const int yr = y + r - 1;
+        hs[r] = 0;
+        if (xin && yr >= 0 && yr < im.H) {
+            const size_t e = (size_t)yr * (size_t)im.W + (size_t)xs;
+            hs[r] = W16 ? (uint32_t)__ldg(reinterpret_cast<const uint16_t *>(im.J) + e) : (uint32_t)__ldg(im.J + e);
+            hs[r] ^= im.flip;
+        }
+    }
+    const int nv = im.W - x;   // pixels of the block's rows inside the image
+    uint32_t cm[4];
+#pragma unroll
+    for (int k = 0; k < 4; k++) cm[k] = (k < nv ? 0xFFFFu : 0u) | (k + 4 < nv ? 0xFFFF0000u : 0u);
+    uint32_t p[4], c[4], n[4];   // rows r - 1, r, r + 1 of J
+    scan_unpack<W16, M>(im, y - 1, x, cm, rj[0], p);
+    scan_unpack<W16, M>(im, y, x, cm, rj[1], c);
+    uint32_t any = 0, nok = 0;
+#pragma unroll
+    for (int r = 0; r < RB; r++) {
+        uint32_t i[4], v[4];
+        scan_unpack<W16, M>(im, y + r + 1, x, cm, rj[r + 2], n);
+        scan_unpack<W16, M>(im, y + r, x, cm, ri[r], i);
+#pragma unroll
+        for (int k = 0; k < 4; k++) v[k] = max3(p[k], c[k], n[k]);
+        // left of word 0 and right of word 3: the adjacent lanes' edge columns or the side halo
+        uint32_t l = __shfl_up_sync(0xffffffffu, CONN == 8 ? v[3] : c[3], 1);
+        uint32_t q = __shfl_down_sync(0xffffffffu, CONN == 8 ? v[0] : c[0], 1);
+        const uint32_t h = CONN == 8 ? max(hs[r], max(hs[r + 1], hs[r + 2])) : hs[r + 1];
+        if (lc == 0) l = h << 16;
+        if (lc == 7) q = h;
+        uint32_t m[4];
+        if (CONN == 8) {
+            m[0] = max3(__byte_perm(l, v[3], 0x5432), v[0], v[1]);
+            m[1] = max3(v[0], v[1], v[2]);
+            m[2] = max3(v[1], v[2], v[3]);
+            m[3] = max3(v[2], v[3], __byte_perm(v[0], q, 0x5432));
+        } else {
+            m[0] = max3(__byte_perm(l, c[3], 0x5432), v[0], c[1]);
+            m[1] = max3(c[0], v[1], c[2]);
+            m[2] = max3(c[1], v[2], c[3]);
+            m[3] = max3(c[2], v[3], __byte_perm(c[0], q, 0x5432));
+        }
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            any |= min2(i[k], m[k]) ^ c[k];
+            nok |= max2(c[k], i[k]) ^ i[k];
+        }
+        if (FEATS && r == 0) {   // the block's first row is a sampled row of the tile
+            static_assert(RB == kFeatRowStep, "a lane block starts on a sampled row");
+            uint32_t nx[4];
+            scan_unpack<W16, M>(im, y + 1, x, cm, ri[1], nx);
+            const bool down = y + 1 < im.H;
+            const uint32_t w0 = __shfl_down_sync(0xffffffffu, i[0], 1);
+            const int nc = min(max(nv, 0), 8);
+            if (y < im.H) {
+                fa.n += (uint32_t)nc;
+                fa.h03 -= (uint32_t)(8 - nc);   // columns outside the image are counted in bin 0 below
+                const uint32_t thr = 16u * ((W16 ? 0xFFFFu : 0xFFu) / 255u);
+#pragma unroll
+                for (int k = 0; k < 4; k++) {
+                    const uint32_t iv = i[k], jv = c[k];
+                    const uint32_t dv = max2(iv, jv) - jv;   // per half max(I - J, 0): no borrow
+                    const uint32_t d8 = W16 ? (dv >> 8) & 0x00FF00FFu : dv;
+                    const uint32_t bl = min(7u, 32u - (uint32_t)__clz(d8 & 0xFFFFu));   // bit length, 0 for 0
+                    const uint32_t bh = min(7u, 32u - (uint32_t)__clz(d8 >> 16));
+                    fa.h03 += (bl < 4 ? 1u << (8 * bl) : 0u) + (bh < 4 ? 1u << (8 * bh) : 0u);
+                    fa.h47 += (bl >= 4 ? 1u << (8 * bl - 32) : 0u) + (bh >= 4 ? 1u << (8 * bh - 32) : 0u);
+                    const uint32_t e = iv ^ jv;
+                    fa.seeds += (uint32_t)((e & 0xFFFFu) == 0 && (jv & 0xFFFFu) != 0) +
+                                (uint32_t)((e >> 16) == 0 && (jv >> 16) != 0);
+                    fa.sI = __dp2a_lo(iv, 0x0101u, fa.sI);
+                    fa.sJ = __dp2a_lo(jv, 0x0101u, fa.sJ);
+                    fa.sD = __dp2a_lo(dv, 0x0101u, fa.sD);
+                    fa.sI2 += (unsigned long long)(iv & 0xFFFFu) * (iv & 0xFFFFu);
+                    fa.sI2 += (unsigned long long)(iv >> 16) * (iv >> 16);
+                    fa.sJ2 += (unsigned long long)(jv & 0xFFFFu) * (jv & 0xFFFFu);
+                    fa.sJ2 += (unsigned long long)(jv >> 16) * (jv >> 16);
+                    // edges: the right neighbours in the tile, the pixel below in the tile
+                    const uint32_t rp = k < 3 ? i[k < 3 ? k + 1 : k] : __byte_perm(i[0], w0, 0x5432);
+                    const uint32_t rm = (k + 1 < nv ? 0xFFFFu : 0u) |
+                                        (k + 5 < nv && (k < 3 || lc < 7) ? 0xFFFF0000u : 0u);
+                    const uint32_t gxv = (max2(iv, rp) - min2(iv, rp)) & rm;
+                    const uint32_t gyv = down ? max2(iv, nx[k]) - min2(iv, nx[k]) : 0u;
+                    fa.edges += (uint32_t)((gxv & 0xFFFFu) + (gyv & 0xFFFFu) > thr) +
+                                (uint32_t)((gxv >> 16) + (gyv >> 16) > thr);
+                }
+            }
+            fa.npix += (uint32_t)(min(max(im.H - y, 0), RB) * nc);
+        }
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            p[k] = c[k];
+            c[k] = n[k];
+        }
+    }
+    can |= any != 0;
+    bad |= nok != 0;
+}
+
+template <bool W16, int CONN, bool FEATS>
+__device__ __forceinline__ void scan_strip_of(const ImageView &im, int y0, int x0, int lane, bool &can, bool &bad,
+                                              FeatAcc &fa) {
+    switch (scan_mode(im, W16, y0, x0)) {   // warp-uniform
+        case kScanSpan: scan_strip<W16, kScanSpan, CONN, FEATS>(im, y0, x0, lane, can, bad, fa); break;
+        case kScanWord: scan_strip<W16, kScanWord, CONN, FEATS>(im, y0, x0, lane, can, bad, fa); break;
+        default: scan_strip<W16, kScanPixel, CONN, FEATS>(im, y0, x0, lane, can, bad, fa); break;
     }
 }
 
-// The streaming scan: warp u of the grid-stride loop takes tile u. FEATS (learned batches):
-// also the tile's 16 features into a.feats (tile t = feature block t).
+// The scan: one strip per warp and step of the grid-stride loop (a strip that can rise marks
+// its tile PENDING); FEATS (learned batches): one tile, whose features (tile t = feature
+// block t) go to a.feats.
 template <typename T, int CONN, bool FEATS>
-__global__ void __launch_bounds__(kThreads, FEATS ? IWPP_STREAM_FEATS_MINB : IWPP_STREAM_MINB)
-    scan_stream_kernel(EngineArgs a) {
+__global__ void __launch_bounds__(kThreads, FEATS ? IWPP_SCAN_FEATS_MINB
+                                                 : (std::is_same<T, AnyPix>::value ? IWPP_SCAN_ANY_MINB : IWPP_SCAN_MINB))
+    scan_block_kernel(EngineArgs a) {
     using RT = RegTile<T, CONN, kCoopStrip>;
+    constexpr int SPT = kCoopRows / kCoopStrip;   // strips per tile
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint64_t nw = (uint64_t)gridDim.x * kWarpsPerCta;
-    for (uint64_t u = (uint64_t)blockIdx.x * kWarpsPerCta + w; u < a.ntiles; u += nw) {
-        const uint32_t t = (uint32_t)u;
+    const uint64_t nw = (uint64_t)gridDim.x * kWarpsPerCta, nu = (uint64_t)a.ntiles * (FEATS ? 1 : SPT);
+    for (uint64_t u = (uint64_t)blockIdx.x * kWarpsPerCta + w; u < nu; u += nw) {
+        const uint32_t t = (uint32_t)(FEATS ? u : u / SPT);
         const long long c0 = clock64();
         const ImageView im = image_of(a, t);
         const uint32_t lt = t - im.tile_base;
         const int ty = (int)(lt / im.tiles_x), tx = (int)(lt % im.tiles_x);
-        const int y0 = ty * kCoopRows, x0 = tx * RT::TW;
-        const int ny = min(kCoopRows, im.H - y0);
+        const int x0 = tx * RT::TW;
+        int y0 = ty * kCoopRows + (FEATS ? 0 : (int)(u % SPT) * kCoopStrip);
+        if (!FEATS && y0 >= im.H) continue;   // a strip below the image (warp-uniform)
         bool can = false, bad = false;
         FeatAcc fa;
-        const bool wide = RT::wide(im), pair = (im.W & 1) == 0;
-        if constexpr (std::is_same<T, AnyPix>::value) {
-            if (wide) {
-                if (pair) scan_tile_stream<true, true, CONN, FEATS>(im, y0, x0, ny, lane, can, bad, fa);
-                else scan_tile_stream<true, false, CONN, FEATS>(im, y0, x0, ny, lane, can, bad, fa);
+        const bool wide = RT::wide(im);
+        for (int s = 0; s < (FEATS ? SPT : 1) && y0 < im.H; s++, y0 += kCoopStrip) {
+            if constexpr (std::is_same<T, AnyPix>::value) {
+                if (wide) scan_strip_of<true, CONN, FEATS>(im, y0, x0, lane, can, bad, fa);
+                else scan_strip_of<false, CONN, FEATS>(im, y0, x0, lane, can, bad, fa);
             } else {
-                if (pair) scan_tile_stream<false, true, CONN, FEATS>(im, y0, x0, ny, lane, can, bad, fa);
-                else scan_tile_stream<false, false, CONN, FEATS>(im, y0, x0, ny, lane, can, bad, fa);
+                scan_strip_of<sizeof(T) == 2, CONN, FEATS>(im, y0, x0, lane, can, bad, fa);
             }
-        } else {
-            if (pair) scan_tile_stream<sizeof(T) == 2, true, CONN, FEATS>(im, y0, x0, ny, lane, can, bad, fa);
-            else scan_tile_stream<sizeof(T) == 2, false, CONN, FEATS>(im, y0, x0, ny, lane, can, bad, fa);
         }
         can = __any_sync(0xffffffffu, can);
         bad = __any_sync(0xffffffffu, bad);
