@@ -27,8 +27,14 @@ struct CoopShared {
     long long c0;                                               // warp 0: the visit's start clock
 };
 
-#ifndef IWPP_CHG_XOR
-#define IWPP_CHG_XOR 1   // 1: passes track "this lane changed something"; a lane that did stores all its rows
+// Chains of rows a pass runs side by side. A row step waits ~50 cycles for the one before it (a
+// shuffle alone takes 24) and the six warps of a scheduler do not always cover that: two chains of
+// 8 rows halve a pass's critical path for ~15 % more passes. 1 -> 2 chains: 512^2 94 -> 86 us,
+// 4096^2 u8 549 -> 516, 3001 x 2777 4-conn 373 -> 347, 4096^2 u16 fill-holes 2515 -> 2223,
+// 16384^2 seeds 9703 -> 9450, 48 uneven images 3477 -> 3346, 256 learned 12680 -> 12608; four
+// chains need too many passes (seeds +12 %).
+#ifndef IWPP_CHAINS
+#define IWPP_CHAINS 2
 #endif
 
 #ifndef IWPP_SCAN_VEC
@@ -118,11 +124,11 @@ __device__ void visit_tile_coop(const EngineArgs &a, const ImageView &im, uint32
     // its current halo
     bool settled = false;
     for (;;) {
-        uint32_t rows = RT::template absorb_side<IWPP_CHG_XOR>(hx, J, I);
+        uint32_t rows = RT::template absorb_side<true>(hx, J, I);
         bool up_fresh = false;   // the strip's last pass was an up pass run with its current halo
         for (;;) {   // joint iterations of the strips
             if (!settled) {
-                const uint32_t chd = RT::template pass_down<IWPP_CHG_XOR>(J, I, jt);
+                const uint32_t chd = RT::template pass_chains<1, IWPP_CHAINS>(J, I, jt);
                 passes++;
                 rows |= chd;
                 // A down pass that changes nothing right after an up pass with the same halo
@@ -131,7 +137,7 @@ __device__ void visit_tile_coop(const EngineArgs &a, const ImageView &im, uint32
                 if (up_fresh && !__any_sync(0xffffffffu, chd != 0)) {
                     settled = true;
                 } else {
-                    const uint32_t chu = RT::template pass_up<IWPP_CHG_XOR>(J, I, jb);
+                    const uint32_t chu = RT::template pass_chains<-1, IWPP_CHAINS>(J, I, jb);
                     passes++;
                     rows |= chu;
                     // likewise an up pass that changes nothing after a down pass with the same
@@ -158,11 +164,9 @@ __device__ void visit_tile_coop(const EngineArgs &a, const ImageView &im, uint32
         if (w == 0 && lane == 0) C.visits++;
         IWPP_CO_MARK(1);
         if (__syncthreads_or(rows != 0)) {
-#if IWPP_CHG_XOR
             // a lane that changed a pixel writes all its rows inside the image
             const int nin = im.H - y0;
             rows = rows == 0 || nin <= 0 ? 0u : (nin >= TH ? 0xFFFFu : (1u << nin) - 1u);
-#endif
             RT::store(im, y0, x0, J, rows, lane);
             RT::notify_scan(s, J, jt, jb, it, ib, lane);
             if (lane == 0) coop_fold_misc(C, s.misc, w);

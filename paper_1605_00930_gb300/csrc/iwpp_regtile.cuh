@@ -403,6 +403,39 @@ struct RegTile {
         return chg;
     }
 
+    // A pass in NCH chains of TH / NCH consecutive rows that advance side by side: the rows of a
+    // chain depend on each other (two shuffles each), those of different chains do not. Rows at a
+    // seam take the other chain's row as it was before the pass, on both sides of every seam
+    // and in both directions, so that a pass that changes nothing after a pass in the other
+    // direction still leaves every pixel checked against all its neighbours. DIR +1: down, halo =
+    // the row above the tile; -1: up, halo = the row below. Returns the OR of the changed bits.
+    template <int DIR, int NCH>
+    static __device__ __forceinline__ uint32_t pass_chains(uint32_t (&J)[TH], const uint32_t (&I)[TH], uint32_t halo) {
+        constexpr int CL = TH / NCH;
+        uint32_t prev[NCH], next[NCH], chg = 0;   // the rows before and after each chain, in pass order
+#pragma unroll
+        for (int q = 0; q < NCH; q++) {   // chain q: rows q CL .. q CL + CL - 1
+            const int before = DIR > 0 ? q * CL - 1 : (q + 1) * CL, after = DIR > 0 ? (q + 1) * CL : q * CL - 1;
+            prev[q] = before < 0 || before >= TH ? halo : J[before < 0 || before >= TH ? 0 : before];
+            next[q] = after < 0 || after >= TH ? 0u : J[after < 0 || after >= TH ? 0 : after];
+        }
+#pragma unroll
+        for (int i = 0; i < CL; i++) {
+#pragma unroll
+            for (int q = 0; q < NCH; q++) {
+                const int r = DIR > 0 ? q * CL + i : q * CL + CL - 1 - i;
+                const uint32_t v = J[r];
+                uint32_t c = i == CL - 1 && NCH > 1 ? max3(v, prev[q], next[q]) : max2(v, prev[q]);
+                if (CONN == 4) c = min2(I[r], c);
+                const uint32_t nv = min2(I[r], hmax_in(c));
+                chg |= nv ^ v;
+                J[r] = nv;
+                prev[q] = nv;
+            }
+        }
+        return chg;
+    }
+
     // ---- raster / anti-raster sweeps (Algorithm 7's scanning phase) ------------------------
     // Along a row, the raster update J(x) <- min(I(x), max(a(x), J(x - 1))) is the map
     // v -> clamp(v, lo, hi) with lo = min(I, a), hi = I, and clamps compose into clamps, so a
