@@ -3,13 +3,21 @@
 //
 // Every pixel carries a site: the background pixel it is nearest to among those its
 // neighbours have offered, packed as (y << 16) | x, or kNoSite. Background pixels are
-// their own sites. A visit holds a 16 x 64 tile in registers (lane c: columns 2c and
-// 2c + 1, one register each per row) and repeats down / up Gauss-Seidel passes in which
-// every pixel takes a neighbour's site if that site is strictly closer to it (the
-// propagation step of Algorithm 8), until a pass pair changes nothing: then no neighbour
-// offers any pixel of the tile a closer site. A halo pixel that one of the tile's sites
-// would bring strictly closer marks its tile for a visit, as in the reconstruction.
+// their own sites. A warp holds a 16 x 64 tile with its halo in shared memory and repeats down /
+// up Gauss-Seidel passes in which every pixel takes a neighbour's site if that site is
+// strictly closer to it (the propagation step of Algorithm 8), until nothing changes: then
+// no neighbour offers any pixel of the tile a closer site. A halo pixel that one of the tile's
+// sites would bring strictly closer marks its tile for a visit, as in the reconstruction.
 // Distances are squared Euclidean, exact in 32-bit integers for sides below 32768.
+//
+// A row step weighs 10 candidates per lane (~150 instructions), so the drain is bound by how many
+// row steps it runs and by how well their instructions are fetched and overlapped. The tile lies in
+// shared memory, not in registers, so that the passes are loops over a row index: the code is a
+// few hundred instructions instead of 2 x 16 unrolled rows (whose fetches were the largest stall),
+// 32 warps fit an SM instead of 8, and rows without foreground, or whose neighbours have not
+// changed, are skipped by bit masks. The distances are written with the sites. Whole call, 4096^2
+// tissue mask (10 % foreground) with distances: 975 us with register tiles and a distance pass
+// (init 33, drain 928, distances 41), 272 us now (0.56 TB/s of its compulsory 9 bytes a pixel).
 #include <cuda_runtime.h>
 
 #include <cstdint>
@@ -37,24 +45,14 @@ __device__ __forceinline__ void offer(int y, int x, uint32_t cand, uint32_t &bes
     bd = take ? d : bd;
 }
 
+// A warp's tile with its one-pixel halo: row y0 + r at index r + 1, column x0 + c at c + 1. The pair
+// of columns 2c - 1, 2c of a row is 8-byte aligned: lane c reads its two pixels and
+// both their horizontal neighbours in two 64-bit accesses.
+constexpr int EPW = ETW + 4;
 struct EdtSmem {
-    uint32_t *hl, *hr;       // ETH + 2: sites of the halo columns, index = row + 1
-    uint32_t *col0, *col63;  // ETH: the tile's first and last column after a solve
-    uint32_t *misc;          // 16: notification flags
+    uint32_t s[ETH + 2][EPW];
 };
-constexpr size_t kEdtWords = 2 * (ETH + 2) + 2 * ETH + 16;
-constexpr size_t kEdtSmemPerWarp = (kEdtWords * 4 + 15) & ~(size_t)15;
-
-__device__ EdtSmem edt_carve(uint8_t *base) {
-    EdtSmem s;
-    uint32_t *w = reinterpret_cast<uint32_t *>(base);
-    s.hl = w; w += ETH + 2;
-    s.hr = w; w += ETH + 2;
-    s.col0 = w; w += ETH;
-    s.col63 = w; w += ETH;
-    s.misc = w;
-    return s;
-}
+constexpr size_t kEdtSmemPerWarp = (sizeof(EdtSmem) + 15) & ~(size_t)15;
 
 __device__ __forceinline__ uint32_t ld_site(const ImageView &im, int y, int x) {
     const bool in = y >= 0 && y < im.H && x >= 0 && x < im.W;
@@ -63,233 +61,250 @@ __device__ __forceinline__ uint32_t ld_site(const ImageView &im, int y, int x) {
     return in ? v : kNoSite;
 }
 
-// The tile (sites, 2 per lane and row) and its halo.
-struct EdtTile {
-    uint32_t e[ETH], o[ETH];   // columns 2c and 2c + 1
-    uint32_t te, to, be, bo;   // halo rows above / below at this lane's columns
+// The rows of work left (bit r: row r): n from the row above, s from the row below, h from
+// the row itself and the side halo. A down pass settles n, an up pass s, either h when it
+// changes nothing.
+struct EdtWork {
+    uint32_t n, s, h;
 };
+constexpr uint32_t kRowBits = (1u << ETH) - 1u;
 
-__device__ void edt_load_halo(const ImageView &im, const EdtSmem &s, int y0, int x0, EdtTile &T, int lane) {
-    const int xe = x0 + 2 * lane;
-    T.te = ld_site(im, y0 - 1, xe);
-    T.to = ld_site(im, y0 - 1, xe + 1);
-    T.be = ld_site(im, y0 + ETH, xe);
-    T.bo = ld_site(im, y0 + ETH, xe + 1);
-    for (int i = lane; i < ETH + 2; i += 32) {
-        s.hl[i] = ld_site(im, y0 + i - 1, x0 - 1);
-        s.hr[i] = ld_site(im, y0 + i - 1, x0 + ETW);
+// Loads the tile and its halo; returns the rows that hold a foreground pixel (only those can
+// change: a background pixel is its own site).
+__device__ uint32_t edt_load(const ImageView &im, EdtSmem &t, int y0, int x0, int lane) {
+    uint32_t fg = 0;
+    uint32_t v0[ETH + 2], v1[ETH + 2];
+#pragma unroll
+    for (int r = 0; r < ETH + 2; r++) {
+        v0[r] = ld_site(im, y0 + r - 1, x0 + lane);
+        v1[r] = ld_site(im, y0 + r - 1, x0 + 32 + lane);
     }
+    const uint32_t hl = ld_site(im, y0 + lane - 1, x0 - 1), hr = ld_site(im, y0 + lane - 1, x0 + ETW);
+#pragma unroll
+    for (int r = 0; r < ETH + 2; r++) {
+        t.s[r][lane + 1] = v0[r];
+        t.s[r][lane + 33] = v1[r];
+        if (r >= 1 && r <= ETH) {
+            const int y = y0 + r - 1;
+            const uint32_t self = ((uint32_t)y << 16) | (uint32_t)(x0 + lane);
+            const bool f = y < im.H && ((x0 + lane < im.W && v0[r] != self) || (x0 + 32 + lane < im.W && v1[r] != self + 32u));
+            if (__any_sync(0xffffffffu, f)) fg |= 1u << (r - 1);
+        }
+    }
+    if (lane < ETH + 2) {
+        t.s[lane][0] = hl;
+        t.s[lane][ETW + 1] = hr;
+    }
+    __syncwarp();
+    return fg;
+}
+
+// The halo again; adds the rows that its changes may change to the work.
+__device__ void edt_reload_halo(const ImageView &im, EdtSmem &t, int y0, int x0, EdtWork &w, int lane) {
+    const uint32_t t0 = ld_site(im, y0 - 1, x0 + lane), t1 = ld_site(im, y0 - 1, x0 + 32 + lane);
+    const uint32_t b0 = ld_site(im, y0 + ETH, x0 + lane), b1 = ld_site(im, y0 + ETH, x0 + 32 + lane);
+    const uint32_t hl = ld_site(im, y0 + lane - 1, x0 - 1), hr = ld_site(im, y0 + lane - 1, x0 + ETW);
+    if (__any_sync(0xffffffffu, t.s[0][lane + 1] != t0 || t.s[0][lane + 33] != t1)) w.n |= 1u;
+    if (__any_sync(0xffffffffu, t.s[ETH + 1][lane + 1] != b0 || t.s[ETH + 1][lane + 33] != b1)) w.s |= 1u << (ETH - 1);
+    t.s[0][lane + 1] = t0;
+    t.s[0][lane + 33] = t1;
+    t.s[ETH + 1][lane + 1] = b0;
+    t.s[ETH + 1][lane + 33] = b1;
+    bool d = false;
+    if (lane < ETH + 2) {
+        d = t.s[lane][0] != hl || t.s[lane][ETW + 1] != hr;
+        t.s[lane][0] = hl;
+        t.s[lane][ETW + 1] = hr;
+    }
+    const uint32_t rows = __ballot_sync(0xffffffffu, d);   // bit r + 1: the halo beside row r changed
+    const uint32_t near = (rows | (rows >> 1) | (rows >> 2)) & kRowBits;   // rows beside and next to it
+    w.h |= near;
+    w.n |= near;
+    w.s |= near;
     __syncwarp();
 }
 
-__device__ void edt_load(const ImageView &im, const EdtSmem &s, int y0, int x0, EdtTile &T, int lane) {
-    const int xe = x0 + 2 * lane;
-#pragma unroll
-    for (int r = 0; r < ETH; r++) {
-        T.e[r] = ld_site(im, y0 + r, xe);
-        T.o[r] = ld_site(im, y0 + r, xe + 1);
-    }
-    edt_load_halo(im, s, y0, x0, T, lane);
-}
-
-// One pass over the rows in the order DIR (+1 down, -1 up): each row from its own sites,
-// the previous row of the pass (already updated) and its horizontal neighbours. Pixels
-// outside the image keep no site. Returns this lane's changed rows.
-template <int CONN, int DIR>
-__device__ __forceinline__ uint32_t edt_pass(const EdtSmem &s, EdtTile &T, int y0, int x0, int H, int W, int lane) {
-    const int xe = x0 + 2 * lane, xo = xe + 1;
-    const bool ve = xe < W, vo = xo < W;
-    uint32_t pe = DIR > 0 ? T.te : T.be, po = DIR > 0 ? T.to : T.bo;   // the row before, this pass
-    uint32_t chg = 0;
-#pragma unroll
-    for (int k = 0; k < ETH; k++) {
-        const int r = DIR > 0 ? k : ETH - 1 - k;
-        const int y = y0 + r;
-        const uint32_t hrow = s.hl[r + 1], hrow_r = s.hr[r + 1];
-        const uint32_t hprev = s.hl[r + 1 - DIR], hprev_r = s.hr[r + 1 - DIR];
-        // horizontal neighbours of this row (values before the pass) and of the previous row
-        uint32_t wo = __shfl_up_sync(0xffffffffu, T.o[r], 1), ee = __shfl_down_sync(0xffffffffu, T.e[r], 1);
-        if (lane == 0) wo = hrow;
-        if (lane == 31) ee = hrow_r;
-        uint32_t pwo = __shfl_up_sync(0xffffffffu, po, 1), pee = __shfl_down_sync(0xffffffffu, pe, 1);
-        if (lane == 0) pwo = hprev;
-        if (lane == 31) pee = hprev_r;
-        // even pixel: own, W, E, and the previous row's N (+ NW, NE)
-        uint32_t be_ = T.e[r], de = site_d2(y, xe, be_);
-        offer(y, xe, wo, be_, de);
-        offer(y, xe, T.o[r], be_, de);
-        offer(y, xe, pe, be_, de);
-        if (CONN == 8) {
-            offer(y, xe, pwo, be_, de);
-            offer(y, xe, po, be_, de);
-        }
-        const bool in = y < H;
-        be_ = (in && ve) ? be_ : kNoSite;
-        // odd pixel: own, W (the even pixel, just updated), E, and the previous row
-        uint32_t bo_ = T.o[r], dd = site_d2(y, xo, bo_);
-        offer(y, xo, be_, bo_, dd);
-        offer(y, xo, ee, bo_, dd);
-        offer(y, xo, po, bo_, dd);
-        if (CONN == 8) {
-            offer(y, xo, pe, bo_, dd);
-            offer(y, xo, pee, bo_, dd);
-        }
-        bo_ = (in && vo) ? bo_ : kNoSite;
-        chg |= (uint32_t)((be_ != T.e[r]) | (bo_ != T.o[r])) << r;
-        T.e[r] = be_;
-        T.o[r] = bo_;
-        pe = be_;
-        po = bo_;
-    }
-    return chg;
-}
-
-// Flag each neighbour one of whose halo pixels a site of the tile would bring strictly
-// closer (misc[(dy + 1) * 3 + dx + 1]).
+// One row from its own sites and the previous row of the pass (DIR +1: the row above). Returns
+// whether a pixel changed (warp-uniform).
 template <int CONN>
-__device__ void edt_notify_scan(const EdtSmem &s, const EdtTile &T, int y0, int x0, int lane) {
-    const int xe = x0 + 2 * lane, xo = xe + 1;
-    if (lane == 0)
-        for (int r = 0; r < ETH; r++) s.col0[r] = T.e[r];
-    if (lane == 31)
-        for (int r = 0; r < ETH; r++) s.col63[r] = T.o[r];
+__device__ __forceinline__ bool edt_row(EdtSmem &t, int r, int dir, int y, int xe, bool ve, bool vo, int lane) {
+    const int xo = xe + 1;
+    uint32_t *row = &t.s[r + 1][2 * lane];
+    const uint32_t *prv = &t.s[r + 1 - dir][2 * lane];
+    const uint2 a = *reinterpret_cast<const uint2 *>(row), b = *reinterpret_cast<const uint2 *>(row + 2);
+    const uint2 pa = *reinterpret_cast<const uint2 *>(prv), pb = *reinterpret_cast<const uint2 *>(prv + 2);
+    // even pixel: own, W, E, and the previous row's N (+ NW, NE)
+    uint32_t be_ = a.y, de = site_d2(y, xe, be_);
+    offer(y, xe, a.x, be_, de);
+    offer(y, xe, b.x, be_, de);
+    offer(y, xe, pa.y, be_, de);
+    if (CONN == 8) {
+        offer(y, xe, pa.x, be_, de);
+        offer(y, xe, pb.x, be_, de);
+    }
+    if (!ve) be_ = kNoSite;
+    // odd pixel: own, W (the even pixel, just updated), E, and the previous row
+    uint32_t bo_ = b.x, dd = site_d2(y, xo, bo_);
+    offer(y, xo, be_, bo_, dd);
+    offer(y, xo, b.y, bo_, dd);
+    offer(y, xo, pb.x, bo_, dd);
+    if (CONN == 8) {
+        offer(y, xo, pa.y, bo_, dd);
+        offer(y, xo, pb.y, bo_, dd);
+    }
+    if (!vo) bo_ = kNoSite;
+    const bool ch = be_ != a.y || bo_ != b.x;
+    const bool any = __any_sync(0xffffffffu, ch);   // (also: every lane has read the row)
+    if (ch) {
+        row[1] = be_;
+        row[2] = bo_;
+    }
+    __syncwarp();
+    return any;
+}
+
+// Passes until the tile is settled; returns the rows that changed. Rows are taken in the order
+// of full down / up passes, less those with nothing to do.
+template <int CONN>
+__device__ uint32_t edt_settle(EdtSmem &t, EdtWork &w, uint32_t fg, int y0, int x0, int W, uint32_t &passes, int lane) {
+    const int xe = x0 + 2 * lane;
+    const bool ve = xe < W, vo = xe + 1 < W;
+    uint32_t rows = 0;
+    while ((w.n | w.s | w.h) & fg) {
+        for (uint32_t left = kRowBits;;) {   // down
+            const uint32_t m = (w.n | w.h) & fg & left;
+            if (m == 0) break;
+            const int r = __ffs(m) - 1;
+            const uint32_t bit = 1u << r;
+            left = ~((bit << 1) - 1u);
+            w.n &= ~bit;
+            w.h &= ~bit;
+            if (edt_row<CONN>(t, r, 1, y0 + r, xe, ve, vo, lane)) {
+                rows |= bit;
+                w.h |= bit;
+                w.n |= bit << 1;
+                w.s |= bit >> 1;
+            }
+        }
+        for (uint32_t left = kRowBits;;) {   // up
+            const uint32_t m = (w.s | w.h) & fg & left;
+            if (m == 0) break;
+            const int r = 31 - __clz(m);
+            const uint32_t bit = 1u << r;
+            left = bit - 1u;
+            w.s &= ~bit;
+            w.h &= ~bit;
+            if (edt_row<CONN>(t, r, -1, y0 + r, xe, ve, vo, lane)) {
+                rows |= bit;
+                w.h |= bit;
+                w.n |= bit << 1;
+                w.s |= bit >> 1;
+            }
+        }
+        passes += 2;
+    }
+    return rows;
+}
+
+// The neighbours one of whose halo pixels a site of the tile would bring strictly closer:
+// bit (dy + 1) * 3 + dx + 1.
+template <int CONN>
+__device__ uint32_t edt_notify_mask(const EdtSmem &t, int y0, int x0, int lane) {
     // halo rows: candidates from the tile's first / last row (the tile's own columns only)
-    bool top = false, bot = false;
+    uint32_t mask = 0;
+#pragma unroll
+    for (int e = 0; e < 2; e++) {
+        const int rt = e ? ETH : 1, rh = e ? ETH + 1 : 0, y = y0 + rh - 1;
+        bool hit = false;
+#pragma unroll
+        for (int q = 0; q < 2; q++) {
+            const int c = 1 + lane + 32 * q, x = x0 + lane + 32 * q;
+            const uint32_t h = t.s[rh][c], d0 = site_d2(y, x, h);
+            uint32_t d = site_d2(y, x, t.s[rt][c]);
+            if (CONN == 8) {
+                if (c > 1) d = min(d, site_d2(y, x, t.s[rt][c - 1]));
+                if (c < ETW) d = min(d, site_d2(y, x, t.s[rt][c + 1]));
+            }
+            hit |= d < d0;
+        }
+        if (__any_sync(0xffffffffu, hit)) mask |= e ? 128u : 2u;
+    }
+    // halo columns: lane -> side (lane / 16) and row (lane % 16)
     {
-        uint32_t wo = __shfl_up_sync(0xffffffffu, T.o[0], 1), ee = __shfl_down_sync(0xffffffffu, T.e[0], 1);
-        uint32_t bwo = __shfl_up_sync(0xffffffffu, T.o[ETH - 1], 1),
-                 bee = __shfl_down_sync(0xffffffffu, T.e[ETH - 1], 1);
-        if (lane == 0) wo = bwo = kNoSite;
-        if (lane == 31) ee = bee = kNoSite;
-        const int yt = y0 - 1, yb = y0 + ETH;
-        uint32_t s1 = T.te, d1 = site_d2(yt, xe, s1), s2 = T.to, d2 = site_d2(yt, xo, s2);
-        const uint32_t d1o = d1, d2o = d2;
-        offer(yt, xe, T.e[0], s1, d1);
-        offer(yt, xo, T.o[0], s2, d2);
+        const int side = lane >> 4, r = lane & 15, y = y0 + r, x = side ? x0 + ETW : x0 - 1;
+        const int ct = side ? ETW : 1, ch = side ? ETW + 1 : 0;
+        uint32_t d = site_d2(y, x, t.s[r + 1][ct]);
         if (CONN == 8) {
-            offer(yt, xe, wo, s1, d1);
-            offer(yt, xe, T.o[0], s1, d1);
-            offer(yt, xo, T.e[0], s2, d2);
-            offer(yt, xo, ee, s2, d2);
+            if (r > 0) d = min(d, site_d2(y, x, t.s[r][ct]));
+            if (r < ETH - 1) d = min(d, site_d2(y, x, t.s[r + 2][ct]));
         }
-        top = (d1 < d1o) || (d2 < d2o);
-        uint32_t s3 = T.be, d3 = site_d2(yb, xe, s3), s4 = T.bo, d4 = site_d2(yb, xo, s4);
-        const uint32_t d3o = d3, d4o = d4;
-        offer(yb, xe, T.e[ETH - 1], s3, d3);
-        offer(yb, xo, T.o[ETH - 1], s4, d4);
-        if (CONN == 8) {
-            offer(yb, xe, bwo, s3, d3);
-            offer(yb, xe, T.o[ETH - 1], s3, d3);
-            offer(yb, xo, T.e[ETH - 1], s4, d4);
-            offer(yb, xo, bee, s4, d4);
-        }
-        bot = (d3 < d3o) || (d4 < d4o);
+        const uint32_t b = __ballot_sync(0xffffffffu, d < site_d2(y, x, t.s[r + 1][ch]));
+        if (b & 0xFFFFu) mask |= 8u;
+        if (b >> 16) mask |= 32u;
     }
-    top = __any_sync(0xffffffffu, top);
-    bot = __any_sync(0xffffffffu, bot);
-    if (lane == 0) {
-        s.misc[1] = top;
-        s.misc[7] = bot;
+    if (CONN == 8) {   // corners: lanes 0..3
+        const int dn = (lane >> 1) & 1, rg = lane & 1;
+        const int y = dn ? y0 + ETH : y0 - 1, x = rg ? x0 + ETW : x0 - 1;
+        const bool hit = lane < 4 && site_d2(y, x, t.s[dn ? ETH : 1][rg ? ETW : 1]) <
+                                         site_d2(y, x, t.s[dn ? ETH + 1 : 0][rg ? ETW + 1 : 0]);
+        const uint32_t b = __ballot_sync(0xffffffffu, hit);
+        mask |= (b & 1u) | ((b & 2u) << 1) | ((b & 4u) << 4) | ((b & 8u) << 5);
     }
-    __syncwarp();
-    // halo columns: one row per lane; corners by lane 0
-    bool lf = false, rt = false;
-    if (lane < ETH) {
-        const int r = lane, y = y0 + r;
-        const int xl = x0 - 1, xr = x0 + ETW;
-        uint32_t sl = s.hl[r + 1], dl = site_d2(y, xl, sl), sr = s.hr[r + 1], dr = site_d2(y, xr, sr);
-        const uint32_t dlo = dl, dro = dr;
-        offer(y, xl, s.col0[r], sl, dl);
-        offer(y, xr, s.col63[r], sr, dr);
-        if (CONN == 8) {
-            if (r > 0) {
-                offer(y, xl, s.col0[r - 1], sl, dl);
-                offer(y, xr, s.col63[r - 1], sr, dr);
-            }
-            if (r < ETH - 1) {
-                offer(y, xl, s.col0[r + 1], sl, dl);
-                offer(y, xr, s.col63[r + 1], sr, dr);
-            }
-        }
-        lf = dl < dlo;
-        rt = dr < dro;
-    }
-    lf = __any_sync(0xffffffffu, lf);
-    rt = __any_sync(0xffffffffu, rt);
-    if (lane == 0) {
-        s.misc[3] = lf;
-        s.misc[5] = rt;
-        uint32_t c0 = 0, c2 = 0, c6 = 0, c8 = 0;
-        if (CONN == 8) {
-            const int yt = y0 - 1, yb = y0 + ETH, xl = x0 - 1, xr = x0 + ETW;
-            c0 = site_d2(yt, xl, s.col0[0]) < site_d2(yt, xl, s.hl[0]);
-            c6 = site_d2(yb, xl, s.col0[ETH - 1]) < site_d2(yb, xl, s.hl[ETH + 1]);
-            c2 = site_d2(yt, xr, s.col63[0]) < site_d2(yt, xr, s.hr[0]);
-            c8 = site_d2(yb, xr, s.col63[ETH - 1]) < site_d2(yb, xr, s.hr[ETH + 1]);
-        }
-        s.misc[0] = c0;
-        s.misc[2] = c2;
-        s.misc[6] = c6;
-        s.misc[8] = c8;
-    }
+    return mask;
 }
 
-__device__ void edt_store(const ImageView &im, int y0, int x0, const EdtTile &T, uint32_t rows, int lane) {
-    const int xe = x0 + 2 * lane;
+// Stores the changed rows' sites and, when asked for (D), their squared distances.
+__device__ void edt_store(const ImageView &im, uint32_t *D, const EdtSmem &t, int y0, int x0, uint32_t rows, int lane) {
     uint32_t *S = reinterpret_cast<uint32_t *>(im.J);
-#pragma unroll
-    for (int r = 0; r < ETH; r++) {
-        if (!((rows >> r) & 1u)) continue;
+    for (uint32_t m = rows; m; m &= m - 1) {
+        const int r = __ffs(m) - 1;
         const size_t row = (size_t)(y0 + r) * im.W;
-        if (xe < im.W) __stcg(S + row + xe, T.e[r]);
-        if (xe + 1 < im.W) __stcg(S + row + xe + 1, T.o[r]);
+#pragma unroll
+        for (int q = 0; q < 2; q++) {
+            const int x = x0 + lane + 32 * q;
+            if (x >= im.W) continue;
+            const uint32_t v = t.s[r + 1][lane + 1 + 32 * q];
+            __stcg(S + row + x, v);
+            if (D) __stcg(D + row + x, site_d2(y0 + r, x, v));
+        }
     }
 }
 
 template <int CONN>
-__device__ void edt_visit(const EngineArgs &a, uint32_t t, uint8_t *wsmem, VisitStats &st, int lane) {
+__device__ void edt_visit(const EngineArgs &a, uint32_t *D, uint32_t t, EdtSmem &sm, VisitStats &st, int lane) {
     const ImageView &im = a.img0;
-    const EdtSmem s = edt_carve(wsmem);
     const int ty = (int)(t / im.tiles_x), tx = (int)(t % im.tiles_x);
     const int y0 = ty * ETH, x0 = tx * ETW;
-    if (lane < 16) s.misc[lane] = 0;
-    EdtTile T;
-    edt_load(im, s, y0, x0, T, lane);
+    const uint32_t fg = edt_load(im, sm, y0, x0, lane);
     uint32_t passes = 0;
+    EdtWork w = {kRowBits, kRowBits, kRowBits};
     for (;;) {
-        uint32_t rows = 0;
-        for (;;) {
-            uint32_t ch = edt_pass<CONN, 1>(s, T, y0, x0, im.H, im.W, lane);
-            ch |= edt_pass<CONN, -1>(s, T, y0, x0, im.H, im.W, lane);
-            passes += 2;
-            rows |= ch;
-            if (!__any_sync(0xffffffffu, ch != 0)) break;
-        }
+        const uint32_t rows = edt_settle<CONN>(sm, w, fg, y0, x0, im.W, passes, lane);
         st.visits++;
-        const bool changed = __any_sync(0xffffffffu, rows != 0);
-        if (changed) {
-            edt_store(im, y0, x0, T, rows, lane);
-            edt_notify_scan<CONN>(s, T, y0, x0, lane);
+        if (rows) {
+            edt_store(im, D, sm, y0, x0, rows, lane);
+            const uint32_t note = edt_notify_mask<CONN>(sm, y0, x0, lane);
             __threadfence();
             __syncwarp();
-        }
-        if (changed && lane < 9 && lane != 4 && s.misc[lane]) {
-            const int ny = ty + lane / 3 - 1, nx = tx + lane % 3 - 1;
-            if (ny >= 0 && nx >= 0 && ny < im.tiles_y && nx < im.tiles_x)
-                notify_tile(a, (uint32_t)(ny * im.tiles_x + nx));
+            if (lane < 9 && lane != 4 && ((note >> lane) & 1u)) {
+                const int ny = ty + lane / 3 - 1, nx = tx + lane % 3 - 1;
+                if (ny >= 0 && nx >= 0 && ny < im.tiles_y && nx < im.tiles_x)
+                    notify_tile(a, (uint32_t)(ny * im.tiles_x + nx));
+            }
         }
         if (!finish_tile(a, t, lane)) break;
         __syncwarp();
-        if (lane < 16) s.misc[lane] = 0;
-        edt_load_halo(im, s, y0, x0, T, lane);
+        edt_reload_halo(im, sm, y0, x0, w, lane);
     }
     st.waves += passes;
 }
 
-// Initialisation (Algorithm 8's first phase): background pixels are their own sites,
-// foreground pixels have none; every tile with a foreground pixel is queued (its first
-// visit takes what its halo offers).
-__global__ void __launch_bounds__(256) edt_init_kernel(EngineArgs a) {
+// Initialisation (Algorithm 8's first phase): background pixels are their own sites (distance
+// 0), foreground pixels have none; every tile with a foreground pixel is queued (its first
+// visit takes what its halo offers). VEC: four pixels per lane and step (the width a multiple
+// of 4, the arrays aligned for it), 8 x 4 + 4 or 8 bytes of a row in flight per lane; else one.
+template <bool VEC>
+__global__ void __launch_bounds__(256) edt_init_kernel(EngineArgs a, uint32_t *D) {
     const ImageView &im = a.img0;
     const int lane = threadIdx.x & 31;
     const uint32_t nw = (gridDim.x * blockDim.x) >> 5;
@@ -298,30 +313,55 @@ __global__ void __launch_bounds__(256) edt_init_kernel(EngineArgs a) {
         const int ty = (int)(t / im.tiles_x), tx = (int)(t % im.tiles_x);
         const int y0 = ty * ETH, x0 = tx * ETW;
         bool fg = false;
-        for (int r = 0; r < ETH; r++) {
-            const int y = y0 + r;
-            if (y >= im.H) break;
+        if (VEC) {
+            const int x = x0 + 4 * (lane & 15);
+            uint32_t m[ETH / 2];
 #pragma unroll
-            for (int q = 0; q < 2; q++) {
-                const int x = x0 + 2 * lane + q;
-                if (x >= im.W) continue;
+            for (int k = 0; k < ETH / 2; k++) {
+                const int y = y0 + 2 * k + (lane >> 4);
+                m[k] = y < im.H && x < im.W ? __ldg(reinterpret_cast<const uint32_t *>(im.I + (size_t)y * im.W + x)) : 0u;
+            }
+#pragma unroll
+            for (int k = 0; k < ETH / 2; k++) {
+                const int y = y0 + 2 * k + (lane >> 4);
+                if (y >= im.H || x >= im.W) continue;
+                fg |= m[k] != 0;
                 const size_t e = (size_t)y * im.W + x;
-                const bool f = im.I[e] != 0;
-                fg |= f;
-                S[e] = f ? kNoSite : ((uint32_t)y << 16) | (uint32_t)x;
+                const uint32_t p = ((uint32_t)y << 16) | (uint32_t)x;
+                const bool f0 = m[k] & 0xFFu, f1 = m[k] & 0xFF00u, f2 = m[k] & 0xFF0000u, f3 = m[k] >> 24;
+                *reinterpret_cast<uint4 *>(S + e) =
+                    make_uint4(f0 ? kNoSite : p, f1 ? kNoSite : p + 1, f2 ? kNoSite : p + 2, f3 ? kNoSite : p + 3);
+                if (D)
+                    *reinterpret_cast<uint4 *>(D + e) = make_uint4(f0 ? kNoSite : 0u, f1 ? kNoSite : 0u, f2 ? kNoSite : 0u,
+                                                                   f3 ? kNoSite : 0u);
+            }
+        } else {
+            for (int r = 0; r < ETH; r++) {
+                const int y = y0 + r;
+                if (y >= im.H) break;
+#pragma unroll
+                for (int q = 0; q < 2; q++) {
+                    const int x = x0 + lane + 32 * q;
+                    if (x >= im.W) continue;
+                    const size_t e = (size_t)y * im.W + x;
+                    const bool f = im.I[e] != 0;
+                    fg |= f;
+                    S[e] = f ? kNoSite : ((uint32_t)y << 16) | (uint32_t)x;
+                    if (D) D[e] = f ? kNoSite : 0u;
+                }
             }
         }
         fg = __any_sync(0xffffffffu, fg);
-        __threadfence();
-        if (lane == 0 && fg) notify_tile(a, t);
+        if (lane == 0 && fg) notify_tile(a, t);   // (the drain is a later kernel: its tiles' sites are visible)
     }
 }
 
+// 8 CTAs (of 4 warps) per SM: 64 registers, 157 KB of shared memory.
 template <int CONN>
-__global__ void __launch_bounds__(kThreads, 2) edt_drain_kernel(EngineArgs a) {
+__global__ void __launch_bounds__(kThreads, 8) edt_drain_kernel(EngineArgs a, uint32_t *D) {
     extern __shared__ __align__(16) uint8_t smem_raw[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    uint8_t *wsmem = smem_raw + warp * kEdtSmemPerWarp;
+    EdtSmem &sm = *reinterpret_cast<EdtSmem *>(smem_raw + warp * kEdtSmemPerWarp);
     VisitStats st = {0, 0, 0, 0};
     unsigned long long idle = 0, busy = 0;
     for (;;) {
@@ -329,18 +369,10 @@ __global__ void __launch_bounds__(kThreads, 2) edt_drain_kernel(EngineArgs a) {
         const uint32_t t = acquire_tile(a, first, idle, lane);
         if (t == kDone) break;
         const unsigned long long b0 = globaltimer_ns();
-        edt_visit<CONN>(a, t, wsmem, st, lane);
+        edt_visit<CONN>(a, D, t, sm, st, lane);
         busy += globaltimer_ns() - b0;
     }
     flush_stats(a, st, idle, busy, lane);
-}
-
-__global__ void edt_dist2_kernel(const uint32_t *S, uint32_t *D, int H, int W) {
-    const size_t n = (size_t)H * W;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        const int y = (int)(i / W), x = (int)(i % W);
-        D[i] = site_d2(y, x, S[i]);
-    }
 }
 
 // Workspace: header (256 B) | tile states | tile-queue ring.
@@ -401,16 +433,18 @@ extern "C" int iwpp_edt(const void *mask, uint32_t *site_out, uint32_t *dist2_ou
     const uint32_t warps_needed = L.ntiles;
     uint32_t ig = (warps_needed + 7) / 8;
     if (ig > (uint32_t)sms * 8) ig = (uint32_t)sms * 8;
-    edt_init_kernel<<<ig, 256, 0, s>>>(a);
+    const bool vec = (W & 3) == 0 && ((uintptr_t)mask & 3) == 0 && ((uintptr_t)site_out & 15) == 0 &&
+                     ((uintptr_t)dist2_out & 15) == 0;
+    if (vec) edt_init_kernel<true><<<ig, 256, 0, s>>>(a, dist2_out);
+    else edt_init_kernel<false><<<ig, 256, 0, s>>>(a, dist2_out);
     const size_t smem = kEdtSmemPerWarp * kWarpsPerCta;
-    void (*drain)(EngineArgs) = connectivity == 8 ? edt_drain_kernel<8> : edt_drain_kernel<4>;
+    void (*drain)(EngineArgs, uint32_t *) = connectivity == 8 ? edt_drain_kernel<8> : edt_drain_kernel<4>;
     int bps = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, drain, kThreads, smem) != cudaSuccess || bps < 1)
         return IWPP_ERR_CUDA;
     long long g = (long long)bps * sms;
     const long long need = ((long long)L.ntiles + kWarpsPerCta - 1) / kWarpsPerCta;
     if (g > need) g = need;
-    drain<<<(int)g, kThreads, smem, s>>>(a);
-    if (dist2_out) edt_dist2_kernel<<<sms * 8, 256, 0, s>>>(site_out, dist2_out, (int)H, (int)W);
+    drain<<<(int)g, kThreads, smem, s>>>(a, dist2_out);
     return cudaGetLastError() == cudaSuccess ? IWPP_OK : IWPP_ERR_CUDA;
 }
