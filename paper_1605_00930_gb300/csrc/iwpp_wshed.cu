@@ -5,12 +5,15 @@
 // Markers are fixed at (gradient, label). A neighbour q offers pixel p the pair
 // (max(level(q), gradient(p)), label(q)) — in the packing, max(v_q, gradient(p) << 16 |
 // label(q)) — and p keeps the smaller of its own pair and every offer. One CTA settles a
-// 64 x 64 tile: each of its four warps holds a 16-row strip in registers (lane c: columns 2c
-// and 2c + 1; the gradient packed as u16x2) and repeats down / up passes of that update; the
-// strips exchange their first and last rows through shared memory between pass pairs until
-// none changes; a halo pixel that the tile's border would improve marks its tile for a visit. The levels reached
-// are unique (the minimax flooding level); which label wins where several reach a pixel at
-// its level depends on the order of work, as in any flooding watershed.
+// 64 x 64 tile held in shared memory with its gradient as eight 8-row strips
+// (iwpp_smemtile.cuh); a halo pixel that the tile's border would improve marks its tile for a
+// visit. The levels reached are unique (the minimax flooding level); which label wins where several
+// reach a pixel at its level depends on the order of work, as in any flooding watershed.
+//
+// A row step weighs ~60 instructions (10 offers of three per lane); what bounds the drain is the
+// number of row steps and the warps there are to overlap them. 2048^2 u16 gradient, 500 markers,
+// 8-connectivity: 1.67 ms with the tile in registers (254 of them, 8 warps per SM, every row in
+// every pass), 1.2 ms now; 4096^2 with 2000 markers 4.6 and 2.9.
 #include <cuda_runtime.h>
 
 #include <cstdint>
@@ -18,52 +21,21 @@
 #include "../../include/iwpp.h"
 #include "iwpp_engine.cuh"
 #include "iwpp_host.h"
+#include "iwpp_smemtile.cuh"
 
 namespace iwpp {
 namespace {
 
 constexpr uint32_t kUnreached = 0xFFFFFFFFu;
-constexpr int WTH = 16, WTW = 64;
-constexpr int WSW = kWarpsPerCta;   // strips per CTA tile
-constexpr int WCH = WTH * WSW;      // CTA tile rows
+constexpr int WTH = kSmStrip, WTW = kSmSide, WSW = kSmWarps, WCH = kSmSide;   // strip rows, tile columns, strips, rows
 
 // The offer of pair v (at a neighbour) to a pixel whose gradient is g (already << 16).
 __device__ __forceinline__ uint32_t offer_ws(uint32_t v, uint32_t g16) { return max(v, g16 | (v & 0xFFFFu)); }
-
-struct WsSmem {
-    uint32_t *hl, *hr;       // WTH + 2: pairs of the halo columns, index = row + 1
-    uint32_t *gl, *gr;       // WTH + 2: their gradient
-    uint32_t *col0, *col63;  // WTH: the tile's first and last column after a solve
-    uint32_t *misc;          // 16: notification flags
-};
-constexpr size_t kWsWords = 4 * (WTH + 2) + 2 * WTH + 16;
-constexpr size_t kWsSmemPerWarp = (kWsWords * 4 + 15) & ~(size_t)15;
-
-__device__ WsSmem ws_carve(uint8_t *base) {
-    WsSmem s;
-    uint32_t *w = reinterpret_cast<uint32_t *>(base);
-    s.hl = w; w += WTH + 2;
-    s.hr = w; w += WTH + 2;
-    s.gl = w; w += WTH + 2;
-    s.gr = w; w += WTH + 2;
-    s.col0 = w; w += WTH;
-    s.col63 = w; w += WTH;
-    s.misc = w;
-    return s;
-}
 
 struct WsArgs {
     const uint32_t *markers;
     const void *grad;
     int u16;
-};
-
-struct WsTile {
-    uint32_t e[WTH], o[WTH];   // pairs of columns 2c, 2c + 1
-    uint32_t g[WTH];           // gradient pair (even low, odd high)
-    uint32_t fixed;            // bit 2r: even pixel of row r fixed, 2r + 1: odd
-    uint32_t te, to, be, bo;   // halo rows' pairs at this lane's columns
-    uint32_t gt, gb;           // their gradient pairs
 };
 
 __device__ __forceinline__ bool inside(const ImageView &im, int y, int x) {
@@ -72,280 +44,92 @@ __device__ __forceinline__ bool inside(const ImageView &im, int y, int x) {
 __device__ __forceinline__ size_t clamp_e(const ImageView &im, int y, int x) {
     return (size_t)min(max(y, 0), im.H - 1) * im.W + min(max(x, 0), im.W - 1);
 }
-__device__ __forceinline__ uint32_t ld_pair_v(const ImageView &im, int y, int x) {
-    const uint32_t v = __ldcg(reinterpret_cast<const uint32_t *>(im.J) + clamp_e(im, y, x));
-    return inside(im, y, x) ? v : kUnreached;
-}
 __device__ __forceinline__ uint32_t ld_grad(const ImageView &im, const WsArgs &w, int y, int x) {
     const size_t e = clamp_e(im, y, x);
-    const uint32_t v = w.u16 ? reinterpret_cast<const uint16_t *>(w.grad)[e] : reinterpret_cast<const uint8_t *>(w.grad)[e];
-    return inside(im, y, x) ? v : 0u;
+    return w.u16 ? (uint32_t)reinterpret_cast<const uint16_t *>(w.grad)[e]
+                 : (uint32_t)reinterpret_cast<const uint8_t *>(w.grad)[e];
 }
 
-__device__ void ws_load_halo(const ImageView &im, const WsArgs &w, const WsSmem &s, int y0, int x0, WsTile &T,
-                             bool with_grad, int lane) {
-    const int xe = x0 + 2 * lane;
-    T.te = ld_pair_v(im, y0 - 1, xe);
-    T.to = ld_pair_v(im, y0 - 1, xe + 1);
-    T.be = ld_pair_v(im, y0 + WTH, xe);
-    T.bo = ld_pair_v(im, y0 + WTH, xe + 1);
-    if (with_grad) {
-        T.gt = ld_grad(im, w, y0 - 1, xe) | (ld_grad(im, w, y0 - 1, xe + 1) << 16);
-        T.gb = ld_grad(im, w, y0 + WTH, xe) | (ld_grad(im, w, y0 + WTH, xe + 1) << 16);
+struct WsOp {
+    using Px = uint32_t;   // (level << 16) | label
+    struct Aux {
+        uint32_t g[kSmSide][kSmSide / 2];    // gradient pairs of the tile (even low, odd high)
+        uint32_t fixed[kSmSide][2];          // per row: lanes whose even / odd pixel is fixed (a marker, or outside)
+        uint32_t hg[4][kSmSide + 2];         // the halo's gradient << 16 per side (all ones outside the image)
+    };
+    using Ctx = WsArgs;
+    static __device__ __forceinline__ Px none() { return kUnreached; }
+    static __device__ __forceinline__ Px load(const ImageView &im, size_t e) {
+        return __ldcg(reinterpret_cast<const uint32_t *>(im.J) + e);
     }
-    for (int i = lane; i < WTH + 2; i += 32) {
-        s.hl[i] = ld_pair_v(im, y0 + i - 1, x0 - 1);
-        s.hr[i] = ld_pair_v(im, y0 + i - 1, x0 + WTW);
-        if (with_grad) {
-            s.gl[i] = ld_grad(im, w, y0 + i - 1, x0 - 1);
-            s.gr[i] = ld_grad(im, w, y0 + i - 1, x0 + WTW);
-        }
+    static __device__ __forceinline__ void store(const ImageView &im, size_t e, Px v) {
+        __stcg(reinterpret_cast<uint32_t *>(im.J) + e, v);
     }
-    __syncwarp();
-}
+    static __device__ __forceinline__ uint32_t halo_aux(const Aux &x, int side, int i) { return x.hg[side][i + 1]; }
+    static __device__ __forceinline__ uint32_t halo_g(const ImageView &im, const Ctx &c, int y, int x) {
+        const uint32_t g = ld_grad(im, c, y, x);
+        return inside(im, y, x) ? g << 16 : 0xFFFFFFFFu;   // an offer there is never an improvement
+    }
 
-__device__ void ws_load(const ImageView &im, const WsArgs &w, const WsSmem &s, int y0, int x0, WsTile &T, int lane) {
-    const int xe = x0 + 2 * lane;
-    T.fixed = 0;
-#pragma unroll
-    for (int r = 0; r < WTH; r++) {
-        const int y = y0 + r;
-        T.e[r] = ld_pair_v(im, y, xe);
-        T.o[r] = ld_pair_v(im, y, xe + 1);
-        T.g[r] = ld_grad(im, w, y, xe) | (ld_grad(im, w, y, xe + 1) << 16);
-        const bool fe = !inside(im, y, xe) || w.markers[clamp_e(im, y, xe)] != 0;
-        const bool fo = !inside(im, y, xe + 1) || w.markers[clamp_e(im, y, xe + 1)] != 0;
-        T.fixed |= ((uint32_t)fe << (2 * r)) | ((uint32_t)fo << (2 * r + 1));
-    }
-    ws_load_halo(im, w, s, y0, x0, T, true, lane);
-}
-
-// One pass (DIR +1 down, -1 up); returns this lane's changed rows.
-template <int CONN, int DIR>
-__device__ __forceinline__ uint32_t ws_pass(const WsSmem &s, WsTile &T, int lane) {
-    uint32_t pe = DIR > 0 ? T.te : T.be, po = DIR > 0 ? T.to : T.bo;
-    uint32_t chg = 0;
-#pragma unroll
-    for (int k = 0; k < WTH; k++) {
-        const int r = DIR > 0 ? k : WTH - 1 - k;
-        uint32_t wo = __shfl_up_sync(0xffffffffu, T.o[r], 1), ee = __shfl_down_sync(0xffffffffu, T.e[r], 1);
-        if (lane == 0) wo = s.hl[r + 1];
-        if (lane == 31) ee = s.hr[r + 1];
-        uint32_t pwo = __shfl_up_sync(0xffffffffu, po, 1), pee = __shfl_down_sync(0xffffffffu, pe, 1);
-        if (lane == 0) pwo = s.hl[r + 1 - DIR];
-        if (lane == 31) pee = s.hr[r + 1 - DIR];
-        const uint32_t ge = T.g[r] << 16, go = T.g[r] & 0xFFFF0000u;
-        uint32_t ne = min(T.e[r], offer_ws(wo, ge));
-        ne = min(ne, offer_ws(T.o[r], ge));
-        ne = min(ne, offer_ws(pe, ge));
-        if (CONN == 8) ne = min(ne, min(offer_ws(pwo, ge), offer_ws(po, ge)));
-        if ((T.fixed >> (2 * r)) & 1u) ne = T.e[r];
-        uint32_t no = min(T.o[r], offer_ws(ne, go));
-        no = min(no, offer_ws(ee, go));
-        no = min(no, offer_ws(po, go));
-        if (CONN == 8) no = min(no, min(offer_ws(pe, go), offer_ws(pee, go)));
-        if ((T.fixed >> (2 * r + 1)) & 1u) no = T.o[r];
-        chg |= (uint32_t)((ne != T.e[r]) | (no != T.o[r])) << r;
-        T.e[r] = ne;
-        T.o[r] = no;
-        pe = ne;
-        po = no;
-    }
-    return chg;
-}
-
-// Flag each neighbour one of whose halo pixels the tile's border would improve.
-template <int CONN>
-__device__ void ws_notify_scan(const WsSmem &s, const WsTile &T, int lane) {
-    if (lane == 0)
-        for (int r = 0; r < WTH; r++) s.col0[r] = T.e[r];
-    if (lane == 31)
-        for (int r = 0; r < WTH; r++) s.col63[r] = T.o[r];
-    bool top = false, bot = false;
-    {
-        uint32_t wo = __shfl_up_sync(0xffffffffu, T.o[0], 1), ee = __shfl_down_sync(0xffffffffu, T.e[0], 1);
-        uint32_t bwo = __shfl_up_sync(0xffffffffu, T.o[WTH - 1], 1),
-                 bee = __shfl_down_sync(0xffffffffu, T.e[WTH - 1], 1);
-        if (lane == 0) wo = bwo = kUnreached;
-        if (lane == 31) ee = bee = kUnreached;
-        const uint32_t gte = T.gt << 16, gto = T.gt & 0xFFFF0000u, gbe = T.gb << 16, gbo = T.gb & 0xFFFF0000u;
-        uint32_t c1 = offer_ws(T.e[0], gte), c2 = offer_ws(T.o[0], gto);
-        uint32_t c3 = offer_ws(T.e[WTH - 1], gbe), c4 = offer_ws(T.o[WTH - 1], gbo);
-        if (CONN == 8) {
-            c1 = min(c1, min(offer_ws(wo, gte), offer_ws(T.o[0], gte)));
-            c2 = min(c2, min(offer_ws(T.e[0], gto), offer_ws(ee, gto)));
-            c3 = min(c3, min(offer_ws(bwo, gbe), offer_ws(T.o[WTH - 1], gbe)));
-            c4 = min(c4, min(offer_ws(T.e[WTH - 1], gbo), offer_ws(bee, gbo)));
-        }
-        top = c1 < T.te || c2 < T.to;
-        bot = c3 < T.be || c4 < T.bo;
-    }
-    top = __any_sync(0xffffffffu, top);
-    bot = __any_sync(0xffffffffu, bot);
-    if (lane == 0) {
-        s.misc[1] = top;
-        s.misc[7] = bot;
-    }
-    __syncwarp();
-    bool lf = false, rt = false;
-    if (lane < WTH) {
-        const int r = lane;
-        const uint32_t gl = s.gl[r + 1] << 16, gr = s.gr[r + 1] << 16;
-        uint32_t cl = offer_ws(s.col0[r], gl), cr = offer_ws(s.col63[r], gr);
-        if (CONN == 8) {
-            if (r > 0) {
-                cl = min(cl, offer_ws(s.col0[r - 1], gl));
-                cr = min(cr, offer_ws(s.col63[r - 1], gr));
-            }
-            if (r < WTH - 1) {
-                cl = min(cl, offer_ws(s.col0[r + 1], gl));
-                cr = min(cr, offer_ws(s.col63[r + 1], gr));
+    static __device__ void load_aux(Aux &x, const ImageView &im, const Ctx &c, int y0, int x0, int w, int lane) {
+        const int xe = x0 + 2 * lane;
+#pragma unroll 8
+        for (int k = 0; k < kSmStrip; k++) {
+            const int r = kSmStrip * w + k, y = y0 + r;
+            const uint32_t ge = ld_grad(im, c, y, xe), go = ld_grad(im, c, y, xe + 1);
+            const bool me = c.markers[clamp_e(im, y, xe)] != 0, mo = c.markers[clamp_e(im, y, xe + 1)] != 0;
+            x.g[r][lane] = ge | (go << 16);
+            const uint32_t fe = __ballot_sync(0xffffffffu, me || !inside(im, y, xe));
+            const uint32_t fo = __ballot_sync(0xffffffffu, mo || !inside(im, y, xe + 1));
+            if (lane == 0) {
+                x.fixed[r][0] = fe;
+                x.fixed[r][1] = fo;
             }
         }
-        lf = cl < s.hl[r + 1];
-        rt = cr < s.hr[r + 1];
-    }
-    lf = __any_sync(0xffffffffu, lf);
-    rt = __any_sync(0xffffffffu, rt);
-    if (lane == 0) {
-        s.misc[3] = lf;
-        s.misc[5] = rt;
-        uint32_t c0 = 0, c2 = 0, c6 = 0, c8 = 0;
-        if (CONN == 8) {
-            c0 = offer_ws(s.col0[0], s.gl[0] << 16) < s.hl[0];
-            c6 = offer_ws(s.col0[WTH - 1], s.gl[WTH + 1] << 16) < s.hl[WTH + 1];
-            c2 = offer_ws(s.col63[0], s.gr[0] << 16) < s.hr[0];
-            c8 = offer_ws(s.col63[WTH - 1], s.gr[WTH + 1] << 16) < s.hr[WTH + 1];
+        {   // side halo: this strip's 16 rows on both sides
+            const int r = kSmStrip * w + lane % kSmStrip, right = lane / kSmStrip % 2;
+            x.hg[right ? kRight : kLeft][r + 1] = halo_g(im, c, y0 + r, right ? x0 + kSmSide : x0 - 1);
         }
-        s.misc[0] = c0;
-        s.misc[2] = c2;
-        s.misc[6] = c6;
-        s.misc[8] = c8;
+        if (w == 0 || w == kSmWarps - 1) {
+            const int side = w == 0 ? kTop : kBottom, y = w == 0 ? y0 - 1 : y0 + kSmSide;
+            for (int i = lane; i < kSmSide + 2; i += 32) x.hg[side][i] = halo_g(im, c, y, x0 + i - 1);
+        }
     }
-}
 
-__device__ void ws_store(const ImageView &im, int y0, int x0, const WsTile &T, uint32_t rows, int lane) {
-    const int xe = x0 + 2 * lane;
-    uint32_t *V = reinterpret_cast<uint32_t *>(im.J);
-#pragma unroll
-    for (int r = 0; r < WTH; r++) {
-        if (!((rows >> r) & 1u)) continue;
-        const size_t row = (size_t)(y0 + r) * im.W;
-        if (xe < im.W) __stcg(V + row + xe, T.e[r]);
-        if (xe + 1 < im.W) __stcg(V + row + xe + 1, T.o[r]);
+    template <int CONN>
+    static __device__ __forceinline__ bool row(const Px *row, const Px *prv, const Aux &x, const Ctx &, int r, int lane,
+                                               Px &e, Px &o) {
+        const uint2 a = *reinterpret_cast<const uint2 *>(row), b = *reinterpret_cast<const uint2 *>(row + 2);
+        const uint2 pa = *reinterpret_cast<const uint2 *>(prv), pb = *reinterpret_cast<const uint2 *>(prv + 2);
+        const uint32_t gp = x.g[r][lane], ge = gp << 16, go = gp & 0xFFFF0000u;
+        const uint32_t fe = x.fixed[r][0], fo = x.fixed[r][1];
+        // (the offers of this row first, those of the row just written last: the shorter chain)
+        uint32_t v = __vimin3_u32(a.y, offer_ws(a.x, ge), offer_ws(b.x, ge));
+        uint32_t u = __vimin3_u32(b.x, offer_ws(b.y, go), offer_ws(pb.x, go));
+        if (CONN == 8) {
+            v = min(v, __vimin3_u32(offer_ws(pa.x, ge), offer_ws(pa.y, ge), offer_ws(pb.x, ge)));
+            u = __vimin3_u32(u, offer_ws(pa.y, go), offer_ws(pb.y, go));
+        } else {
+            v = min(v, offer_ws(pa.y, ge));
+        }
+        e = (fe >> lane) & 1u ? a.y : v;
+        o = (fo >> lane) & 1u ? b.x : min(u, offer_ws(e, go));
+        return e != a.y || o != b.x;
     }
-}
-
-// The CTA tile's shared state: each strip's first and last row (even and odd pair per lane),
-// the tile's notification flags, the popped tile.
-struct WsShared {
-    uint32_t rows[WSW][4][32];
-    uint32_t misc[16];
-    uint32_t tile, redo;
+    static __device__ __forceinline__ bool changes(Px h, uint32_t g16, const Px (&q)[3], int n) {
+        uint32_t v = offer_ws(q[0], g16);
+        if (n > 1) v = __vimin3_u32(v, offer_ws(q[1], g16), offer_ws(q[2], g16));
+        return v < h;
+    }
+    static __device__ __forceinline__ bool changes_own(Px v, const Aux &x, const Ctx &, int r, int c, const Px (&q)[3],
+                                                       int n) {
+        if ((x.fixed[r][c & 1] >> (c >> 1)) & 1u) return false;
+        const uint32_t gp = x.g[r][c >> 1];
+        return changes(v, (c & 1) ? gp & 0xFFFF0000u : gp << 16, q, n);
+    }
 };
-constexpr size_t kWsSmemCta = kWsSmemPerWarp * WSW + sizeof(WsShared);
 
-// Fold one strip's notification flags into the CTA tile's (a strip's top / bottom side is the
-// tile's only for the first / last strip; its corners beside the tile's inner rows lie in the
-// west / east neighbours).
-__device__ __forceinline__ void ws_fold_misc(WsShared &C, const uint32_t *m, int w) {
-    if (w == 0) {
-        atomicOr(&C.misc[0], m[0]);
-        atomicOr(&C.misc[1], m[1]);
-        atomicOr(&C.misc[2], m[2]);
-    } else {
-        atomicOr(&C.misc[3], m[0]);
-        atomicOr(&C.misc[5], m[2]);
-    }
-    if (w == WSW - 1) {
-        atomicOr(&C.misc[6], m[6]);
-        atomicOr(&C.misc[7], m[7]);
-        atomicOr(&C.misc[8], m[8]);
-    } else {
-        atomicOr(&C.misc[3], m[6]);
-        atomicOr(&C.misc[5], m[8]);
-    }
-    atomicOr(&C.misc[3], m[3]);
-    atomicOr(&C.misc[5], m[5]);
-}
-
-// One visit of CTA tile t by the whole CTA (every thread calls it with the same t), including
-// the re-processing rounds when the tile is notified while the CTA holds it.
-template <int CONN>
-__device__ void ws_visit(const EngineArgs &a, const WsArgs &wa, uint32_t t, uint8_t *wsmem, WsShared &C,
-                         VisitStats &st, int w, int lane) {
-    const ImageView &im = a.img0;
-    const WsSmem s = ws_carve(wsmem);
-    const int ty = (int)(t / im.tiles_x), tx = (int)(t % im.tiles_x);
-    const int y0 = ty * WCH + WTH * w, x0 = tx * WTW;
-    if (lane < 16) s.misc[lane] = 0;
-    if (threadIdx.x < 16) C.misc[threadIdx.x] = 0;
-    WsTile T;
-    ws_load(im, wa, s, y0, x0, T, lane);
-    uint32_t passes = 0;
-    for (;;) {
-        uint32_t rows = 0;
-        bool active = true;
-        for (;;) {   // joint iterations of the strips
-            uint32_t ch = 0;
-            if (active) {
-                ch = ws_pass<CONN, 1>(s, T, lane);
-                ch |= ws_pass<CONN, -1>(s, T, lane);
-                passes += 2;
-                rows |= ch;
-            }
-            C.rows[w][0][lane] = T.e[0];
-            C.rows[w][1][lane] = T.o[0];
-            C.rows[w][2][lane] = T.e[WTH - 1];
-            C.rows[w][3][lane] = T.o[WTH - 1];
-            __syncthreads();
-            uint32_t nte = T.te, nto = T.to, nbe = T.be, nbo = T.bo;
-            if (w > 0) {
-                nte = C.rows[w - 1][2][lane];
-                nto = C.rows[w - 1][3][lane];
-            }
-            if (w < WSW - 1) {
-                nbe = C.rows[w + 1][0][lane];
-                nbo = C.rows[w + 1][1][lane];
-            }
-            const bool halo = __any_sync(0xffffffffu, nte != T.te || nto != T.to || nbe != T.be || nbo != T.bo);
-            T.te = nte;
-            T.to = nto;
-            T.be = nbe;
-            T.bo = nbo;
-            active = halo || __any_sync(0xffffffffu, ch != 0);
-            if (!__syncthreads_or(active)) break;
-        }
-        if (w == 0 && lane == 0) st.visits++;
-        if (__syncthreads_or(rows != 0)) {
-            ws_store(im, y0, x0, T, rows, lane);
-            ws_notify_scan<CONN>(s, T, lane);
-            if (lane == 0) ws_fold_misc(C, s.misc, w);
-            __threadfence();
-            __syncthreads();
-            if (w == 0 && lane < 9 && lane != 4 && C.misc[lane]) {
-                const int ny = ty + lane / 3 - 1, nx = tx + lane % 3 - 1;
-                if (ny >= 0 && nx >= 0 && ny < im.tiles_y && nx < im.tiles_x)
-                    notify_tile(a, (uint32_t)(ny * im.tiles_x + nx));
-            }
-        }
-        if (w == 0) {
-            const bool r = finish_tile(a, t, lane);
-            if (lane == 0) C.redo = r;
-        }
-        __syncthreads();
-        const bool redo = C.redo != 0;
-        if (!redo) break;
-        // re-process: the strips stay in registers; only the tile's halo can have changed
-        if (lane < 16) s.misc[lane] = 0;
-        if (threadIdx.x < 16) C.misc[threadIdx.x] = 0;
-        ws_load_halo(im, wa, s, y0, x0, T, false, lane);
-        __syncthreads();
-    }
-    st.waves += passes;
-}
-
-// Initialisation, one warp per 16 x 64 strip: markers take (gradient, label), everything else
+// Initialisation, one warp per 8 x 64 strip: markers take (gradient, label), everything else
 // is unreached; the CTA tile of every strip holding a marker is queued. Labels above 65534
 // stop the call with IWPP_ERR_ARG.
 __global__ void __launch_bounds__(256) ws_init_kernel(EngineArgs a, WsArgs w, uint32_t nstrips) {
@@ -381,29 +165,13 @@ __global__ void __launch_bounds__(256) ws_init_kernel(EngineArgs a, WsArgs w, ui
     }
 }
 
+#ifndef IWPP_WS_MINB
+#define IWPP_WS_MINB 3   // CTAs (of 8 warps) per SM: 80 registers; 4 (64) are 8 % faster on 4096^2, 10 % slower on 2048^2
+#endif
 template <int CONN>
-__global__ void __launch_bounds__(kThreads, 2) ws_drain_kernel(EngineArgs a, WsArgs wa) {
+__global__ void __launch_bounds__(kSmThreads, IWPP_WS_MINB) ws_drain_kernel(EngineArgs a, WsArgs wa) {
     extern __shared__ __align__(16) uint8_t smem_raw[];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    uint8_t *wsmem = smem_raw + warp * kWsSmemPerWarp;
-    WsShared &C = *reinterpret_cast<WsShared *>(smem_raw + WSW * kWsSmemPerWarp);
-    VisitStats st = {0, 0, 0, 0};
-    unsigned long long idle = 0, busy = 0;
-    for (;;) {
-        if (warp == 0) {
-            bool first;
-            const uint32_t t = acquire_tile(a, first, idle, lane);
-            if (lane == 0) C.tile = t;
-        }
-        __syncthreads();
-        const uint32_t t = C.tile;
-        if (t == kDone) break;
-        const unsigned long long b0 = globaltimer_ns();
-        ws_visit<CONN>(a, wa, t, wsmem, C, st, warp, lane);
-        if (warp == 0) busy += globaltimer_ns() - b0;
-        __syncthreads();   // every warp has read C.tile before the next pop overwrites it
-    }
-    flush_stats(a, st, idle, busy, lane);
+    sm_drain<WsOp, CONN>(a, wa, *reinterpret_cast<SmemTile<WsOp> *>(smem_raw));
 }
 
 // labels in place (0 where unreached), levels optionally (-1 where unreached)
@@ -417,7 +185,7 @@ __global__ void ws_finish_kernel(uint32_t *V, int32_t *levels, size_t n) {
 
 struct WsLayout {
     size_t state, queue, total;
-    uint32_t ntiles, nstrips;   // 64 x 64 CTA tiles; 16 x 64 strips
+    uint32_t ntiles, nstrips;   // 64 x 64 CTA tiles; 8 x 64 strips
     int tiles_x, tiles_y;
 };
 
@@ -484,14 +252,17 @@ extern "C" int iwpp_watershed(const uint32_t *markers, const void *gradient, int
     uint32_t ig = (L.nstrips + 7) / 8;
     if (ig > (uint32_t)sms * 8) ig = (uint32_t)sms * 8;
     ws_init_kernel<<<ig, 256, 0, s>>>(a, w, L.nstrips);
-    const size_t smem = kWsSmemCta;
+    const size_t smem = sizeof(SmemTile<WsOp>);
     void (*drain)(EngineArgs, WsArgs) = connectivity == 8 ? ws_drain_kernel<8> : ws_drain_kernel<4>;
     int bps = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, drain, kThreads, smem) != cudaSuccess || bps < 1)
+    if (cudaFuncSetAttribute((const void *)drain, cudaFuncAttributePreferredSharedMemoryCarveout,
+                             cudaSharedmemCarveoutMaxShared) != cudaSuccess)
+        return IWPP_ERR_CUDA;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, drain, kSmThreads, smem) != cudaSuccess || bps < 1)
         return IWPP_ERR_CUDA;
     long long g = (long long)bps * sms;
     if (g > (long long)L.ntiles) g = L.ntiles;   // one CTA per tile
-    drain<<<(int)g, kThreads, smem, s>>>(a, w);
+    drain<<<(int)g, kSmThreads, smem, s>>>(a, w);
     const size_t n = (size_t)H * (size_t)W;
     ws_finish_kernel<<<sms * 8, 256, 0, s>>>(labels_out, levels_out, n);
     return cudaGetLastError() == cudaSuccess ? IWPP_OK : IWPP_ERR_CUDA;
