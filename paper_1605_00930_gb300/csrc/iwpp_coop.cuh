@@ -123,27 +123,31 @@ __device__ void visit_tile_coop(const EngineArgs &a, const ImageView &im, uint32
     // settled: the strip is a fixed point of J <- min(I, max over the neighbourhood) for
     // its current halo
     bool settled = false;
+    uint32_t sum = RT::value_sum(J);   // of this lane's pixels: a pass changed one when it changes
     for (;;) {
-        uint32_t rows = RT::template absorb_side<true>(hx, J, I);
+        const uint32_t sum0 = sum;
+        RT::absorb_side(hx, J, I);
         bool up_fresh = false;   // the strip's last pass was an up pass run with its current halo
         for (;;) {   // joint iterations of the strips
             if (!settled) {
-                const uint32_t chd = RT::template pass_chains<1, IWPP_CHAINS>(J, I, jt);
+                const uint32_t sd = RT::template pass_chains<1, IWPP_CHAINS>(J, I, jt);
+                const bool chd = sd != sum;   // (a round's first: the halo absorbed before it too)
+                sum = sd;
                 passes++;
-                rows |= chd;
                 // A down pass that changes nothing right after an up pass with the same halo
                 // leaves every pixel checked, with final values, against its neighbours below
                 // (by the up pass) and above and beside it (by the down pass): settled.
-                if (up_fresh && !__any_sync(0xffffffffu, chd != 0)) {
+                if (up_fresh && !__any_sync(0xffffffffu, chd)) {
                     settled = true;
                 } else {
-                    const uint32_t chu = RT::template pass_chains<-1, IWPP_CHAINS>(J, I, jb);
+                    const uint32_t su = RT::template pass_chains<-1, IWPP_CHAINS>(J, I, jb);
+                    const bool chu = su != sum;
+                    sum = su;
                     passes++;
-                    rows |= chu;
                     // likewise an up pass that changes nothing after a down pass with the same
                     // halo (a strip that changed may still be short of its fixed point: its
                     // next pass finds out, measured cheaper than a residual check here)
-                    settled = !__any_sync(0xffffffffu, chu != 0);
+                    settled = !__any_sync(0xffffffffu, chu);
                     up_fresh = true;
                 }
             }
@@ -163,10 +167,10 @@ __device__ void visit_tile_coop(const EngineArgs &a, const ImageView &im, uint32
         }
         if (w == 0 && lane == 0) C.visits++;
         IWPP_CO_MARK(1);
-        if (__syncthreads_or(rows != 0)) {
+        if (__syncthreads_or(sum != sum0)) {
             // a lane that changed a pixel writes all its rows inside the image
             const int nin = im.H - y0;
-            rows = rows == 0 || nin <= 0 ? 0u : (nin >= TH ? 0xFFFFu : (1u << nin) - 1u);
+            const uint32_t rows = sum == sum0 || nin <= 0 ? 0u : (nin >= TH ? 0xFFFFu : (1u << nin) - 1u);
             RT::store(im, y0, x0, J, rows, lane);
             RT::notify_scan(s, J, jt, jb, it, ib, lane);
             if (lane == 0) coop_fold_misc(C, s.misc, w);

@@ -341,8 +341,7 @@ struct RegTile {
 
     // Raise the side columns' pixels by what the side halo offers them: J <- min(I, max(J, halo
     // pixels beside it)). The halo is fixed while the tile is being settled, so doing it once
-    // leaves the side halo out of every row step of the passes. Returns as the passes do.
-    template <bool DIFF = false>
+    // leaves the side halo out of every row step of the passes. Returns this lane's mask of changed rows.
     static __device__ __forceinline__ uint32_t absorb_side(const uint32_t *hx, uint32_t (&J)[TH],
                                                            const uint32_t (&I)[TH]) {
         uint32_t chg = 0, h0 = hx[0], h1 = hx[1];
@@ -350,8 +349,7 @@ struct RegTile {
         for (int r = 0; r < TH; r++) {
             const uint32_t h2 = CONN == 8 || r + 2 <= TH ? hx[r + 2] : 0u;
             const uint32_t nv = min2(I[r], CONN == 8 ? max2(J[r], max3(h0, h1, h2)) : max2(J[r], h1));
-            if (DIFF) chg |= nv ^ J[r];
-            else chg |= (uint32_t)(nv != J[r]) << r;
+            chg |= (uint32_t)(nv != J[r]) << r;
             J[r] = nv;
             h0 = h1;
             h1 = h2;
@@ -408,16 +406,21 @@ struct RegTile {
     // seam take the other chain's row as it was before the pass, on both sides of every seam
     // and in both directions, so that a pass that changes nothing after a pass in the other
     // direction still leaves every pixel checked against all its neighbours. DIR +1: down, halo =
-    // the row above the tile; -1: up, halo = the row below. Returns the OR of the changed bits.
+    // the row above the tile; -1: up, halo = the row below. Returns the sum of the lane's pixels
+    // (value_sum): values never fall, so a pass changed a pixel exactly when the sum is another. The sum
+    // is one dp2a per row, which issues beside the min / max / permute pipe that bounds a
+    // pass (measured), where an OR of the changed bits took that pipe's slots: 12 -> 10 of its
+    // cycles per row.
     template <int DIR, int NCH>
     static __device__ __forceinline__ uint32_t pass_chains(uint32_t (&J)[TH], const uint32_t (&I)[TH], uint32_t halo) {
         constexpr int CL = TH / NCH;
-        uint32_t prev[NCH], next[NCH], chg = 0;   // the rows before and after each chain, in pass order
+        uint32_t prev[NCH], next[NCH], sum[NCH];   // the rows before and after each chain, in pass order
 #pragma unroll
         for (int q = 0; q < NCH; q++) {   // chain q: rows q CL .. q CL + CL - 1
             const int before = DIR > 0 ? q * CL - 1 : (q + 1) * CL, after = DIR > 0 ? (q + 1) * CL : q * CL - 1;
             prev[q] = before < 0 || before >= TH ? halo : J[before < 0 || before >= TH ? 0 : before];
             next[q] = after < 0 || after >= TH ? 0u : J[after < 0 || after >= TH ? 0 : after];
+            sum[q] = 0;
         }
 #pragma unroll
         for (int i = 0; i < CL; i++) {
@@ -428,12 +431,22 @@ struct RegTile {
                 uint32_t c = i == CL - 1 && NCH > 1 ? max3(v, prev[q], next[q]) : max2(v, prev[q]);
                 if (CONN == 4) c = min2(I[r], c);
                 const uint32_t nv = min2(I[r], hmax_in(c));
-                chg |= nv ^ v;
+                sum[q] = __dp2a_lo(nv, 0x0101u, sum[q]);
                 J[r] = nv;
                 prev[q] = nv;
             }
         }
-        return chg;
+        uint32_t total = 0;
+#pragma unroll
+        for (int q = 0; q < NCH; q++) total += sum[q];
+        return total;
+    }
+    // Sum of the lane's pixels (below 2^22).
+    static __device__ __forceinline__ uint32_t value_sum(const uint32_t (&J)[TH]) {
+        uint32_t s = 0;
+#pragma unroll
+        for (int r = 0; r < TH; r++) s = __dp2a_lo(J[r], 0x0101u, s);
+        return s;
     }
 
     // ---- raster / anti-raster sweeps (Algorithm 7's scanning phase) ------------------------
