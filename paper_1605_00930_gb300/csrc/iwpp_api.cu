@@ -121,7 +121,7 @@ static cudaError_t ensure_smem_attr(int shape, int v, size_t bytes) {
     const int want = (int)(bytes < 100 * 1024 ? 100 * 1024 : bytes);
     cudaError_t e;
     for (void (*f)(EngineArgs) : {k.scan, k.drain, k.reg.scan, k.reg.drain, k.reg.drain_hi, k.coop.scan, k.coop.drain,
-                                  k.coop.scan_sweeps, k.coop.scan_feats}) {
+                                  k.coop.drain_hi, k.coop.scan_sweeps, k.coop.scan_feats}) {
         if (!f) continue;
         e = cudaFuncSetAttribute((const void *)f, cudaFuncAttributeMaxDynamicSharedMemorySize, want);
         if (e != cudaSuccess) return e;
@@ -142,8 +142,8 @@ int device_sm_count() {
 // The scan and persistent kernels of a plan (queue or register local solver) and their
 // shared memory. Register plans asking for more than kRegBlocks CTAs per SM get the
 // high-occupancy build of the persistent kernel.
-static void (*drain_fn(const iwpp_plan &p, const KernelSet &k))(EngineArgs) {
-    if (p.local_solver == IWPP_SOLVER_COOP) return k.coop.drain;
+static void (*drain_fn(const iwpp_plan &p, const KernelSet &k, bool hi = false))(EngineArgs) {
+    if (p.local_solver == IWPP_SOLVER_COOP) return hi ? k.coop.drain_hi : k.coop.drain;
     if (p.local_solver != IWPP_SOLVER_REGISTER) return k.drain;
     return p.blocks_per_sm > kRegBlocks ? k.reg.drain_hi : k.reg.drain;
 }
@@ -170,7 +170,7 @@ static int tiles_per_cta(const iwpp_plan &p) { return p.local_solver == IWPP_SOL
 
 // Persistent CTAs for a plan: blocks_per_sm (or the occupancy maximum) x SMs, never more
 // CTAs than needed to give every tile its own warp.
-static int drain_grid(const iwpp_plan &p, int v, uint32_t ntiles) {
+static int drain_grid(const iwpp_plan &p, int v, uint32_t ntiles, bool hi = false) {
     const int shape = shape_index(p.tile_h, p.tile_w);
     if (shape < 0) return 0;
     const KernelSet &k = kernels(shape, v);
@@ -179,7 +179,7 @@ static int drain_grid(const iwpp_plan &p, int v, uint32_t ntiles) {
     if (ensure_smem_attr(shape, v, k.smem ? k.smem((uint32_t)p.smem_queue_cap) : smem) != cudaSuccess) return 0;
     int bps = p.blocks_per_sm;
     if (bps <= 0) {
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, drain_fn(p, k), kThreads, smem) != cudaSuccess)
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, drain_fn(p, k, hi), kThreads, smem) != cudaSuccess)
             return 0;
         if (bps <= 0) return 0;
     }
@@ -357,7 +357,13 @@ int reconstruct_one(void *marker, const void *mask, int64_t H, int64_t W, int co
             a.defer_push = 0;
         }
     }
-    if (phases & kPhaseDrain) drain_fn(p, k)<<<L.grid, kThreads, drain_smem(p, k), stream>>>(a);
+    if (phases & kPhaseDrain) {
+        const bool hi = p.local_solver == IWPP_SOLVER_COOP && p.blocks_per_sm == 0 && op == IWPP_DILATE &&
+                        L.ntiles >= kCoopHiTiles;
+        const int grid = hi ? drain_grid(p, v, L.ntiles, true) : L.grid;
+        if (grid <= 0) return IWPP_ERR_CUDA;
+        drain_fn(p, k, hi)<<<grid, kThreads, drain_smem(p, k), stream>>>(a);
+    }
     return cudaGetLastError() == cudaSuccess ? IWPP_OK : IWPP_ERR_CUDA;
 }
 

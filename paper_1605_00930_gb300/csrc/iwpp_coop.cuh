@@ -21,6 +21,7 @@ struct CoopShared {
     uint32_t rows[kWarpsPerCta][2][32];   // each strip's first and last row, per lane
     uint32_t misc[16];                    // the CTA tile's notification values (3 x 3 grid)
     uint32_t tile, redo;
+    uint32_t k16;                         // 65536 (RegTile::hmax_in)
     // Run statistics, kept here rather than in registers that would stay live through every
     // visit's passes (measured: fewer spills, drains 2-3 % faster); flushed at the end.
     unsigned long long k0, idle, visits, waves[kWarpsPerCta];   // start time, pop waits (warp 0), visits, passes
@@ -98,9 +99,10 @@ __device__ __forceinline__ void coop_fold_misc(CoopShared &C, const uint32_t *m,
 
 // One visit of CTA tile t by the whole CTA (every thread calls it with the same t), including
 // the re-processing rounds when the tile is notified while the CTA holds it.
-template <typename T, int CONN>
+template <typename T, int CONN, bool HI = false>
 __device__ void visit_tile_coop(const EngineArgs &a, const ImageView &im, uint32_t t, uint8_t *wsmem,
                                 CoopShared &C, unsigned long long *ph, int w, int lane) {
+    const uint32_t k16 = HI ? C.k16 : 0u;
     (void)ph;
 #if IWPP_PHASE_TIMING
     long long pt = clock64();
@@ -130,7 +132,7 @@ __device__ void visit_tile_coop(const EngineArgs &a, const ImageView &im, uint32
         bool up_fresh = false;   // the strip's last pass was an up pass run with its current halo
         for (;;) {   // joint iterations of the strips
             if (!settled) {
-                const uint32_t sd = RT::template pass_chains<1, IWPP_CHAINS>(J, I, jt);
+                const uint32_t sd = RT::template pass_chains<1, IWPP_CHAINS, HI>(J, I, jt, k16);
                 const bool chd = sd != sum;   // (a round's first: the halo absorbed before it too)
                 sum = sd;
                 passes++;
@@ -140,7 +142,7 @@ __device__ void visit_tile_coop(const EngineArgs &a, const ImageView &im, uint32
                 if (up_fresh && !__any_sync(0xffffffffu, chd)) {
                     settled = true;
                 } else {
-                    const uint32_t su = RT::template pass_chains<-1, IWPP_CHAINS>(J, I, jb);
+                    const uint32_t su = RT::template pass_chains<-1, IWPP_CHAINS, HI>(J, I, jb, k16);
                     const bool chu = su != sum;
                     sum = su;
                     passes++;
@@ -208,7 +210,7 @@ __device__ void visit_tile_coop(const EngineArgs &a, const ImageView &im, uint32
 }
 
 // One CTA tile visit, dispatched on the tile's image kind (CTA-uniform: one tile per CTA).
-template <typename T, int CONN, bool MIXED>
+template <typename T, int CONN, bool MIXED, bool HI>
 __device__ __forceinline__ void visit_tile_coop_any(const EngineArgs &a, uint32_t t, uint8_t *wsmem, CoopShared &C,
                                                     unsigned long long *ph, int w, int lane) {
 #if IWPP_PHASE_TIMING
@@ -219,7 +221,7 @@ __device__ __forceinline__ void visit_tile_coop_any(const EngineArgs &a, uint32_
     if (w == 0) ph[7] += (unsigned long long)(clock64() - c0);
 #endif
     if (!MIXED) {
-        visit_tile_coop<T, CONN>(a, im, t, wsmem, C, ph, w, lane);
+        visit_tile_coop<T, CONN, HI>(a, im, t, wsmem, C, ph, w, lane);
         return;
     }
     switch (im.kind) {
@@ -235,11 +237,15 @@ __device__ __forceinline__ void visit_tile_coop_any(const EngineArgs &a, uint32_
 // visit variants inlined, keeps 4 CTAs per SM (at 5 it spills). The builds for one pixel
 // type take kCoopBlocks (single images: more CTAs slow the images bound by one chain of
 // tile hops), the build for u8 + u16 batches kCoopBatchBlocks (a batch keeps every worker
-// busy, so the seventh CTA pays despite its spills). Without a plan's blocks_per_sm the
-// grid is the occupancy the launch bounds give.
-template <typename T, int CONN, bool MIXED>
+// busy, so the seventh CTA pays despite its spills). HI: the build for large single dilations,
+// kCoopHiBlocks CTAs per SM with the permutes of a row step as multiply-adds: with that many tiles per
+// worker the issue of the row steps is what counts, not their latency (16384^2 seeds 9.00 -> 8.57 ms,
+// 8192^2 h-dome 1248 -> 1204 us; 4096^2 u16 fill-holes, a chain of tile hops, 2.22 -> 2.33 ms).
+// Without a plan's blocks_per_sm the grid is the occupancy the launch bounds give.
+template <typename T, int CONN, bool MIXED, bool HI = false>
 __global__ void __launch_bounds__(kThreads, MIXED ? kRegBlocks
-                                                 : (std::is_same<T, AnyPix>::value ? kCoopBatchBlocks : kCoopBlocks))
+                                                 : (HI ? kCoopHiBlocks
+                                                       : (std::is_same<T, AnyPix>::value ? kCoopBatchBlocks : kCoopBlocks)))
     drain_coop_kernel(EngineArgs a) {
     using RT = RegTile<T, CONN, kCoopStrip>;
     extern __shared__ __align__(16) uint8_t smem_raw[];
@@ -252,6 +258,7 @@ __global__ void __launch_bounds__(kThreads, MIXED ? kRegBlocks
         C.k0 = globaltimer_ns();
         C.idle = 0;
         C.visits = 0;
+        C.k16 = 65536u;
     }
     for (;;) {
         if (warp == 0) {
@@ -262,7 +269,7 @@ __global__ void __launch_bounds__(kThreads, MIXED ? kRegBlocks
         __syncthreads();
         const uint32_t t = C.tile;
         if (t == kDone) break;
-        visit_tile_coop_any<T, CONN, MIXED>(a, t, wsmem, C, ph, warp, lane);
+        visit_tile_coop_any<T, CONN, MIXED, HI>(a, t, wsmem, C, ph, warp, lane);
         __syncthreads();   // every warp has read C.tile before the next pop overwrites it
     }
     if (lane == 0) {   // passes of every strip; visits and times of warp 0 (busy: the rest of the run)

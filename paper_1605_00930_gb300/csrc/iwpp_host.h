@@ -32,6 +32,12 @@ constexpr int kCoopBlocks = IWPP_COOP_MINB;   // CTAs per SM of the cooperative 
 #define IWPP_COOP_BATCH_MINB 7   // its build for u8 + u16 batches (72 registers, ~250 B of spills)
 #endif
 constexpr int kCoopBatchBlocks = IWPP_COOP_BATCH_MINB;
+// Its build for single dilations of at least kCoopHiTiles tiles (drain_hi). Measured, 6 CTAs per SM
+// -> this build: 4096 tiles h-dome 468 -> 467 us, 8836 tiles 718 -> 700 (seeds 1744 -> 1750), 16384
+// tiles 1248 -> 1204 (seeds 2173 -> 2115), 36864 tiles u16 2650 -> 2520, 65536 tiles seeds 9000 -> 8565;
+// erosions (fill-holes) are bound by tile hops up to the largest size and lose 3-5 %.
+constexpr int kCoopHiBlocks = 7;
+constexpr uint32_t kCoopHiTiles = 8192;
 RegKernelSet reg_kernel_set(int th, int tw, int v);
 RegKernelSet coop_kernel_set(int th, int tw, int v);   // cooperative solver (64 x 64 tiles)
 

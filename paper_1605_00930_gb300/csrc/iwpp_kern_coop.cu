@@ -18,7 +18,8 @@ static RegKernelSet coop_set() {
     if constexpr (MIXED || !IWPP_SCAN_BLOCK) k.scan = scan_strip_coop_kernel<T, CONN, MIXED>;
     else k.scan = scan_block_kernel<T, CONN, false>;
     k.drain = drain_coop_kernel<T, CONN, MIXED>;
-    k.drain_hi = nullptr;   // one build of the persistent kernel
+    if constexpr (MIXED || std::is_same<T, AnyPix>::value) k.drain_hi = nullptr;   // batches: one build
+    else k.drain_hi = drain_coop_kernel<T, CONN, MIXED, true>;
     k.smem = &coop_smem_fn<T, CONN>;
     k.scan_sweeps = scan_coop_kernel<T, CONN, MIXED, true>;
     // features in the scan: not for the mixed-kind build

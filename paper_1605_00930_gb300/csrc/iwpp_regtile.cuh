@@ -339,6 +339,16 @@ struct RegTile {
         return max3(v, left_of(p, v), right_of(v, n));
     }
 
+    // The same with the multiply pipe doing part of the pairing: the pair is shifted once, the shifted
+    // word is what goes up, and each side is one multiply-add (k16 = 65536, a value the compiler
+    // does not know, or it would shift on the busy pipe) instead of a permute: 2 of 10 cycles of that
+    // pipe less per row, for 4 cycles more latency.
+    static __device__ __forceinline__ uint32_t hmax_in(uint32_t v, uint32_t k16) {
+        const uint32_t x = v >> 16;
+        const uint32_t p = __shfl_up_sync(0xffffffffu, x, 1), n = __shfl_down_sync(0xffffffffu, v, 1);
+        return max3(v, v * k16 + p, n * k16 + x);
+    }
+
     // Raise the side columns' pixels by what the side halo offers them: J <- min(I, max(J, halo
     // pixels beside it)). The halo is fixed while the tile is being settled, so doing it once
     // leaves the side halo out of every row step of the passes. Returns this lane's mask of changed rows.
@@ -410,9 +420,10 @@ struct RegTile {
     // (value_sum): values never fall, so a pass changed a pixel exactly when the sum is another. The sum
     // is one dp2a per row, which issues beside the min / max / permute pipe that bounds a
     // pass (measured), where an OR of the changed bits took that pipe's slots: 12 -> 10 of its
-    // cycles per row.
-    template <int DIR, int NCH>
-    static __device__ __forceinline__ uint32_t pass_chains(uint32_t (&J)[TH], const uint32_t (&I)[TH], uint32_t halo) {
+    // cycles per row. MULADD: pair the neighbours by multiply-adds (k16).
+    template <int DIR, int NCH, bool MULADD>
+    static __device__ __forceinline__ uint32_t pass_chains(uint32_t (&J)[TH], const uint32_t (&I)[TH], uint32_t halo,
+                                                           uint32_t k16) {
         constexpr int CL = TH / NCH;
         uint32_t prev[NCH], next[NCH], sum[NCH];   // the rows before and after each chain, in pass order
 #pragma unroll
@@ -430,7 +441,7 @@ struct RegTile {
                 const uint32_t v = J[r];
                 uint32_t c = i == CL - 1 && NCH > 1 ? max3(v, prev[q], next[q]) : max2(v, prev[q]);
                 if (CONN == 4) c = min2(I[r], c);
-                const uint32_t nv = min2(I[r], hmax_in(c));
+                const uint32_t nv = min2(I[r], MULADD ? hmax_in(c, k16) : hmax_in(c));
                 sum[q] = __dp2a_lo(nv, 0x0101u, sum[q]);
                 J[r] = nv;
                 prev[q] = nv;
