@@ -164,7 +164,7 @@ IWPP_API int iwpp_reconstruct_plan(void *marker_inout, const void *mask, int64_t
  * (precondition check, `plan->sweeps` tile-local raster / anti-raster sweep pairs
  * of Algorithm 7, and frontier initialisation: the tiles whose pixels can still
  * be raised are queued — with one FIFO (value_levels <= 1) in a spread order that
- * keeps tiles next to each other apart in the queue, by two small kernels after the
+ * keeps tiles next to each other apart in the queue, by a small kernel after the
  * scan); iwpp_drain then runs the persistent kernel that drains
  * the queued tiles (Algorithm 7's irregular propagation phase). Calling
  * iwpp_scan and then iwpp_drain with identical arguments on one stream is exactly

@@ -334,9 +334,8 @@ int reconstruct_one(void *marker, const void *mask, int64_t H, int64_t W, int co
     if (ensure_smem_attr(shape, v, smem) != cudaSuccess) return IWPP_ERR_CUDA;
 
     if (phases & kPhaseScan) {
-        // header, tile states, level counters
-        if (cudaMemsetAsync(base, 0, L.queue, stream) != cudaSuccess) return IWPP_ERR_CUDA;
-        if (cudaMemsetAsync(base + L.queue, 0xFF, (size_t)L.ntiles * 4 * L.nlevels, stream) != cudaSuccess)
+        // header, tile states, level counters, queue slots
+        if (cudaMemsetAsync(base, 0, L.queue + (size_t)L.ntiles * 4 * L.nlevels, stream) != cudaSuccess)
             return IWPP_ERR_CUDA;
         const int sms = device_sm_count();
         const uint32_t ctas = (L.ntiles + kWarpsPerCta - 1) / kWarpsPerCta;
@@ -352,8 +351,7 @@ int reconstruct_one(void *marker, const void *mask, int64_t H, int64_t W, int co
         if (spread) {
             const uint32_t cgrid = (L.ntiles + 255) / 256 < (uint32_t)(sms * 8) ? (L.ntiles + 255) / 256
                                                                                  : (uint32_t)(sms * 8);
-            compact_kernel<<<cgrid, 256, 0, stream>>>(a);
-            finalize_queue_kernel<<<cgrid, 256, 0, stream>>>(a);
+            queue_spread_kernel<<<cgrid, 256, 0, stream>>>(a);
             a.defer_push = 0;
         }
     }
@@ -521,8 +519,9 @@ int reconstruct_batch(const iwpp_image *imgs, int n, const iwpp_plan *plan_in, c
         tile_image_kernel<<<g, 256, 0, stream>>>(table, n, reinterpret_cast<uint32_t *>(base + L.timg));
     }
     if (cudaMemsetAsync(base, 0, 256, stream) != cudaSuccess) return IWPP_ERR_CUDA;
-    if (cudaMemsetAsync(base + L.state, 0, (size_t)L.ntiles * 4, stream) != cudaSuccess) return IWPP_ERR_CUDA;
-    if (cudaMemsetAsync(base + L.queue, 0xFF, (size_t)L.ntiles * 4, stream) != cudaSuccess) return IWPP_ERR_CUDA;
+    // tile states and queue slots (adjacent)
+    if (cudaMemsetAsync(base + L.state, 0, L.queue - L.state + (size_t)L.ntiles * 4, stream) != cudaSuccess)
+        return IWPP_ERR_CUDA;
     const int sms = device_sm_count();
     const uint32_t ctas = (L.ntiles + kWarpsPerCta - 1) / kWarpsPerCta;
     const uint32_t scan_grid = ctas < (uint32_t)(sms * 16) ? ctas : (uint32_t)(sms * 16);

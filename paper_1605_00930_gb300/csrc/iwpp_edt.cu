@@ -426,8 +426,7 @@ extern "C" int iwpp_edt(const void *mask, uint32_t *site_out, uint32_t *dist2_ou
     a.ntiles = L.ntiles;
     a.watchdog_ns = 10ll * 1000 * 1000 * 1000;
     a.nlevels = 1;
-    if (cudaMemsetAsync(base, 0, L.queue, s) != cudaSuccess) return IWPP_ERR_CUDA;
-    if (cudaMemsetAsync(base + L.queue, 0xFF, (size_t)L.ntiles * 4, s) != cudaSuccess) return IWPP_ERR_CUDA;
+    if (cudaMemsetAsync(base, 0, L.queue + (size_t)L.ntiles * 4, s) != cudaSuccess) return IWPP_ERR_CUDA;
     const int sms = device_sm_count();
     if (sms <= 0) return IWPP_ERR_CUDA;
     const uint32_t warps_needed = L.ntiles;

@@ -235,8 +235,7 @@ extern "C" int iwpp_skiz(const uint32_t *markers, const uint8_t *mask, uint32_t 
     a.ntiles = L.ntiles;
     a.watchdog_ns = 10ll * 1000 * 1000 * 1000;
     a.nlevels = 1;
-    if (cudaMemsetAsync(base, 0, L.queue, s) != cudaSuccess) return IWPP_ERR_CUDA;
-    if (cudaMemsetAsync(base + L.queue, 0xFF, (size_t)L.ntiles * 4, s) != cudaSuccess) return IWPP_ERR_CUDA;
+    if (cudaMemsetAsync(base, 0, L.queue + (size_t)L.ntiles * 4, s) != cudaSuccess) return IWPP_ERR_CUDA;
     const int sms = device_sm_count();
     if (sms <= 0) return IWPP_ERR_CUDA;
     uint32_t ig = (L.nstrips + 7) / 8;

@@ -245,8 +245,7 @@ extern "C" int iwpp_watershed(const uint32_t *markers, const void *gradient, int
     w.markers = markers;
     w.grad = gradient;
     w.u16 = dtype == IWPP_U16;
-    if (cudaMemsetAsync(base, 0, L.queue, s) != cudaSuccess) return IWPP_ERR_CUDA;
-    if (cudaMemsetAsync(base + L.queue, 0xFF, (size_t)L.ntiles * 4, s) != cudaSuccess) return IWPP_ERR_CUDA;
+    if (cudaMemsetAsync(base, 0, L.queue + (size_t)L.ntiles * 4, s) != cudaSuccess) return IWPP_ERR_CUDA;
     const int sms = device_sm_count();
     if (sms <= 0) return IWPP_ERR_CUDA;
     uint32_t ig = (L.nstrips + 7) / 8;
