@@ -237,7 +237,7 @@ __device__ __forceinline__ void visit_tile_coop_any(const EngineArgs &a, uint32_
 // visit variants inlined, keeps 4 CTAs per SM (at 5 it spills). The builds for one pixel
 // type take kCoopBlocks (single images: more CTAs slow the images bound by one chain of
 // tile hops), the build for u8 + u16 batches kCoopBatchBlocks (a batch keeps every worker
-// busy, so the seventh CTA pays despite its spills). HI: the build for large single dilations,
+// busy, so the seventh CTA pays despite its few spills). HI: the build for large single dilations,
 // kCoopHiBlocks CTAs per SM with the permutes of a row step as multiply-adds: with that many tiles per
 // worker the issue of the row steps is what counts, not their latency (16384^2 seeds 9.00 -> 8.57 ms,
 // 8192^2 h-dome 1248 -> 1204 us; 4096^2 u16 fill-holes, a chain of tile hops, 2.22 -> 2.33 ms).

