@@ -82,29 +82,26 @@ struct SkOp {
     static __device__ __forceinline__ uint32_t halo_aux(const Aux &, int, int) { return 0; }
 
     template <int CONN>
-    static __device__ __forceinline__ bool row(const Px *row, const Px *prv, const Aux &, const Ctx &, int, int, Px &e,
-                                               Px &o) {
-        const ulonglong2 a = *reinterpret_cast<const ulonglong2 *>(row), b = *reinterpret_cast<const ulonglong2 *>(row + 2);
-        const ulonglong2 pa = *reinterpret_cast<const ulonglong2 *>(prv),
-                         pb = *reinterpret_cast<const ulonglong2 *>(prv + 2);
+    static __device__ __forceinline__ bool row(const Px (&q)[4], const Px (&p)[4], const Aux &, const Ctx &, int, int,
+                                               Px &e, Px &o) {
         uint32_t m, lc;
         if (CONN == 8) {
-            const Px q[5] = {a.x, b.x, pa.x, pa.y, pb.x};
-            join(q, m, lc);
+            const Px c[5] = {q[0], q[2], p[0], p[1], p[2]};
+            join(c, m, lc);
         } else {
-            const Px q[3] = {a.x, b.x, pa.y};
-            join(q, m, lc);
+            const Px c[3] = {q[0], q[2], p[1]};
+            join(c, m, lc);
         }
-        e = pack(accept(unpack(a.y), m, lc));
+        e = pack(accept(unpack(q[1]), m, lc));
         if (CONN == 8) {
-            const Px q[5] = {e, b.y, pa.y, pb.x, pb.y};
-            join(q, m, lc);
+            const Px c[5] = {e, q[3], p[1], p[2], p[3]};
+            join(c, m, lc);
         } else {
-            const Px q[3] = {e, b.y, pb.x};
-            join(q, m, lc);
+            const Px c[3] = {e, q[3], p[2]};
+            join(c, m, lc);
         }
-        o = pack(accept(unpack(b.x), m, lc));
-        return e != a.y || o != b.x;
+        o = pack(accept(unpack(q[2]), m, lc));
+        return e != q[1] || o != q[2];
     }
     static __device__ __forceinline__ bool changes(Px h, uint32_t, const Px (&q)[3], int n) {
         const Px c[3] = {q[0], n > 1 ? q[1] : none(), n > 2 ? q[2] : none()};

@@ -18,15 +18,16 @@
 // 1500 / 3119 / 1316 / 591, (8, pair) 1122 / 2946 / 1171 / 423, (8, single pass) 1432 / 2974 / 1217 / 458,
 // (16, pair) 1324 / 4011 / 1767 / 440. Against one warp's 16 rows in registers: 1541 / 4565 / 3252 / 1135.
 //
-// Strips read the adjacent strips' boundary rows where they lie; a pixel is written by its own
-// strip only, in one aligned access, and pixels only ever improve, so a row read while it changes is a
-// valid older or newer state, and the strip whose row changed hands its neighbour the row again
-// at the next barrier.
+// Strips read the adjacent strips' boundary rows where they lie. A pixel is written by its own strip
+// only; between two barriers those writes, and the reads of another strip's row, are single relaxed
+// accesses of a whole pixel (sm_st_relaxed, sm_ld_relaxed): a pixel read while it changes is its
+// older or its newer state, never half of each, and pixels only ever improve, so either is
+// valid; the strip whose row changed hands its neighbour the row again at the next barrier.
 //
 // Op: the operator. Px (a pixel's state, one aligned 4- or 8-byte word), Aux (what it needs
 // beside it) and Ctx (kernel arguments), none() (outside the image), load / store, load_aux,
-// row<CONN> (one lane's two pixels of a row step), halo_aux and changes (whether pixels
-// offered to a halo pixel change it).
+// row<CONN> (one lane's two pixels of a row step, from columns 2c - 1 .. 2c + 2 of the row and of the
+// one before it), halo_aux and changes (whether pixels offered to a halo pixel change it).
 #pragma once
 #include "iwpp_engine.cuh"
 
@@ -54,6 +55,33 @@ struct SmemTile {
 struct RowWork {
     uint32_t n, s, h;
 };
+
+// One whole pixel of shared memory, relaxed at block scope.
+__device__ __forceinline__ uint32_t sm_ld_relaxed(const uint32_t *p) {
+    uint32_t v;
+    asm volatile("ld.relaxed.cta.shared.u32 %0, [%1];" : "=r"(v) : "r"((uint32_t)__cvta_generic_to_shared(p)) : "memory");
+    return v;
+}
+__device__ __forceinline__ unsigned long long sm_ld_relaxed(const unsigned long long *p) {
+    unsigned long long v;
+    asm volatile("ld.relaxed.cta.shared.u64 %0, [%1];" : "=l"(v) : "r"((uint32_t)__cvta_generic_to_shared(p)) : "memory");
+    return v;
+}
+__device__ __forceinline__ void sm_st_relaxed(uint32_t *p, uint32_t v) {
+    asm volatile("st.relaxed.cta.shared.u32 [%0], %1;" ::"r"((uint32_t)__cvta_generic_to_shared(p)), "r"(v) : "memory");
+}
+__device__ __forceinline__ void sm_st_relaxed(unsigned long long *p, unsigned long long v) {
+    asm volatile("st.relaxed.cta.shared.u64 [%0], %1;" ::"r"((uint32_t)__cvta_generic_to_shared(p)), "l"(v) : "memory");
+}
+// Four pixels of a row of the warp's own strip or of the halo, from an even index on.
+__device__ __forceinline__ void sm_ld4(const uint32_t *p, uint32_t (&q)[4]) {
+    const uint2 a = *reinterpret_cast<const uint2 *>(p), b = *reinterpret_cast<const uint2 *>(p + 2);
+    q[0] = a.x; q[1] = a.y; q[2] = b.x; q[3] = b.y;
+}
+__device__ __forceinline__ void sm_ld4(const unsigned long long *p, unsigned long long (&q)[4]) {
+    const ulonglong2 a = *reinterpret_cast<const ulonglong2 *>(p), b = *reinterpret_cast<const ulonglong2 *>(p + 2);
+    q[0] = a.x; q[1] = a.y; q[2] = b.x; q[3] = b.y;
+}
 
 template <class Op>
 __device__ __forceinline__ typename Op::Px sm_ld(const ImageView &im, int y, int x) {
@@ -151,12 +179,19 @@ __device__ uint32_t sm_pass_pair(SmemTile<Op> &S, const typename Op::Ctx &ctx, R
             const int ri = kSmStrip * w + r + 1;
             typename Op::Px *row = &S.v[ri][2 * lane];
             const typename Op::Px *prv = &S.v[ri - dir][2 * lane];
-            typename Op::Px e, o;
-            const bool ch = Op::template row<CONN>(row, prv, S.aux, ctx, ri - 1, lane, e, o);
+            typename Op::Px q[4], p[4], e, o;
+            sm_ld4(row, q);
+            if (dir > 0 ? r == 0 && w > 0 : r == kSmStrip - 1 && w < kSmWarps - 1) {   // another strip's row
+#pragma unroll
+                for (int i = 0; i < 4; i++) p[i] = sm_ld_relaxed(prv + i);
+            } else {
+                sm_ld4(prv, p);
+            }
+            const bool ch = Op::template row<CONN>(q, p, S.aux, ctx, ri - 1, lane, e, o);
             const bool any = __any_sync(0xffffffffu, ch);   // (also: every lane has read the row)
             if (ch) {
-                row[1] = e;
-                row[2] = o;
+                sm_st_relaxed(row + 1, e);
+                sm_st_relaxed(row + 2, o);
             }
             __syncwarp();
             if (any) {

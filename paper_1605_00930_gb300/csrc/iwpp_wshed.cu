@@ -97,24 +97,22 @@ struct WsOp {
     }
 
     template <int CONN>
-    static __device__ __forceinline__ bool row(const Px *row, const Px *prv, const Aux &x, const Ctx &, int r, int lane,
-                                               Px &e, Px &o) {
-        const uint2 a = *reinterpret_cast<const uint2 *>(row), b = *reinterpret_cast<const uint2 *>(row + 2);
-        const uint2 pa = *reinterpret_cast<const uint2 *>(prv), pb = *reinterpret_cast<const uint2 *>(prv + 2);
+    static __device__ __forceinline__ bool row(const Px (&q)[4], const Px (&p)[4], const Aux &x, const Ctx &, int r,
+                                               int lane, Px &e, Px &o) {
         const uint32_t gp = x.g[r][lane], ge = gp << 16, go = gp & 0xFFFF0000u;
         const uint32_t fe = x.fixed[r][0], fo = x.fixed[r][1];
         // (the offers of this row first, those of the row just written last: the shorter chain)
-        uint32_t v = __vimin3_u32(a.y, offer_ws(a.x, ge), offer_ws(b.x, ge));
-        uint32_t u = __vimin3_u32(b.x, offer_ws(b.y, go), offer_ws(pb.x, go));
+        uint32_t v = __vimin3_u32(q[1], offer_ws(q[0], ge), offer_ws(q[2], ge));
+        uint32_t u = __vimin3_u32(q[2], offer_ws(q[3], go), offer_ws(p[2], go));
         if (CONN == 8) {
-            v = min(v, __vimin3_u32(offer_ws(pa.x, ge), offer_ws(pa.y, ge), offer_ws(pb.x, ge)));
-            u = __vimin3_u32(u, offer_ws(pa.y, go), offer_ws(pb.y, go));
+            v = min(v, __vimin3_u32(offer_ws(p[0], ge), offer_ws(p[1], ge), offer_ws(p[2], ge)));
+            u = __vimin3_u32(u, offer_ws(p[1], go), offer_ws(p[3], go));
         } else {
-            v = min(v, offer_ws(pa.y, ge));
+            v = min(v, offer_ws(p[1], ge));
         }
-        e = (fe >> lane) & 1u ? a.y : v;
-        o = (fo >> lane) & 1u ? b.x : min(u, offer_ws(e, go));
-        return e != a.y || o != b.x;
+        e = (fe >> lane) & 1u ? q[1] : v;
+        o = (fo >> lane) & 1u ? q[2] : min(u, offer_ws(e, go));
+        return e != q[1] || o != q[2];
     }
     static __device__ __forceinline__ bool changes(Px h, uint32_t g16, const Px (&q)[3], int n) {
         uint32_t v = offer_ws(q[0], g16);
