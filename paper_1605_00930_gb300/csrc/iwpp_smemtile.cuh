@@ -105,7 +105,9 @@ __device__ void sm_load(const ImageView &im, SmemTile<Op> &S, int y0, int x0, in
 // changes may change are added to the work.
 template <class Op, bool RELOAD>
 __device__ void sm_load_halo(const ImageView &im, SmemTile<Op> &S, int y0, int x0, RowWork &k, int w, int lane) {
-    const int r = lane % kSmStrip, right = lane / kSmStrip % 2;   // this lane's pixel of the side halo
+    // this lane's pixel of the side halo (those of lanes from 2 kSmStrip on repeat and are not used)
+    const int r = lane % kSmStrip, right = lane / kSmStrip % 2;
+    const bool side = lane < 2 * kSmStrip;
     const int ri = kSmStrip * w + r + 1, ci = right ? kSmSide + 1 : 0;
     const typename Op::Px sv = sm_ld<Op>(im, y0 + kSmStrip * w + r, right ? x0 + kSmSide : x0 - 1);
     const bool outer = w == 0 || w == kSmWarps - 1;
@@ -117,7 +119,7 @@ __device__ void sm_load_halo(const ImageView &im, SmemTile<Op> &S, int y0, int x
         c = sm_ld<Op>(im, yh, (lane & 1) ? x0 + kSmSide : x0 - 1);
     }
     if (RELOAD) {
-        const uint32_t d = __ballot_sync(0xffffffffu, S.v[ri][ci] != sv);
+        const uint32_t d = __ballot_sync(0xffffffffu, side && S.v[ri][ci] != sv);
         const uint32_t rows = (d | (d >> kSmStrip)) & kSmRows;
         const uint32_t near = (rows | (rows << 1) | (rows >> 1)) & kSmRows;   // beside or next to a changed pixel
         k.n |= near;
@@ -137,7 +139,7 @@ __device__ void sm_load_halo(const ImageView &im, SmemTile<Op> &S, int y0, int x
             }
         }
     }
-    S.v[ri][ci] = sv;
+    if (side) S.v[ri][ci] = sv;
     if (outer) {
         S.v[rh][lane + 1] = a;
         S.v[rh][lane + 33] = b;

@@ -86,7 +86,7 @@ struct WsOp {
                 x.fixed[r][1] = fo;
             }
         }
-        {   // side halo: this strip's 16 rows on both sides
+        if (lane < 2 * kSmStrip) {   // side halo: this strip's rows on both sides
             const int r = kSmStrip * w + lane % kSmStrip, right = lane / kSmStrip % 2;
             x.hg[right ? kRight : kLeft][r + 1] = halo_g(im, c, y0 + r, right ? x0 + kSmSide : x0 - 1);
         }
