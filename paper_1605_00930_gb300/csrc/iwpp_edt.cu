@@ -154,7 +154,8 @@ __device__ __forceinline__ bool edt_row(EdtSmem &t, int r, int dir, int y, int x
     }
     if (!vo) bo_ = kNoSite;
     const bool ch = be_ != a.y || bo_ != b.x;
-    const bool any = __any_sync(0xffffffffu, ch);   // (also: every lane has read the row)
+    const bool any = __any_sync(0xffffffffu, ch);
+    __syncwarp();   // every lane has read the row
     if (ch) {
         row[1] = be_;
         row[2] = bo_;

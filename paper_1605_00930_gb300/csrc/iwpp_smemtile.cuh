@@ -190,7 +190,8 @@ __device__ uint32_t sm_pass_pair(SmemTile<Op> &S, const typename Op::Ctx &ctx, R
                 sm_ld4(prv, p);
             }
             const bool ch = Op::template row<CONN>(q, p, S.aux, ctx, ri - 1, lane, e, o);
-            const bool any = __any_sync(0xffffffffu, ch);   // (also: every lane has read the row)
+            const bool any = __any_sync(0xffffffffu, ch);
+            __syncwarp();   // every lane has read the row
             if (ch) {
                 sm_st_relaxed(row + 1, e);
                 sm_st_relaxed(row + 2, o);
