@@ -10,14 +10,20 @@
 // sites would bring strictly closer marks its tile for a visit, as in the reconstruction.
 // Distances are squared Euclidean, exact in 32-bit integers for sides below 32768.
 //
-// A row step weighs 10 candidates per lane (~150 instructions), so the drain is bound by how many
-// row steps it runs and by how well their instructions are fetched and overlapped. The tile lies in
-// shared memory, not in registers, so that the passes are loops over a row index: the code is a
-// few hundred instructions instead of 2 x 16 unrolled rows (whose fetches were the largest stall),
-// 32 warps fit an SM instead of 8, and rows without foreground, or whose neighbours have not
-// changed, are skipped by bit masks. The distances are written with the sites. Whole call, 4096^2
-// tissue mask (10 % foreground) with distances: 975 us with register tiles and a distance pass
-// (init 33, drain 928, distances 41), 272 us now (0.56 TB/s of its compulsory 9 bytes a pixel).
+// Large images are bound by how many row steps are run and by how well their instructions are
+// fetched and overlapped, small ones (fewer tiles than the 4864 resident warps) and long chains of tiles by the
+// latency of a row step and of a visit's loads and stores. The tile lies in shared memory, not in
+// registers, so that the passes are loops over a row index: the code is a few hundred instructions
+// instead of 2 x 16 unrolled rows (whose fetches were the largest stall), 32 warps fit an SM
+// instead of 8, and rows without foreground, or whose neighbours have not changed, are skipped by
+// bit masks. For the latency, rows that follow one another are a run (edt_pass), a row step takes minima
+// of three (edt_step), and a visit's loads and stores go out together. The distances are written
+// with the sites. Whole calls with distances, microseconds: register tiles of 220 registers and a
+// distance pass / shared tiles with each row through shared memory and ten offers in turn / now:
+//   tissue (10 % foreground), 8-connectivity: 4096^2 965 / 266 / 256, 512^2 155 / 80 / 68, 200^2 71 / 45 / 37;
+//   4-connectivity: 4096^2 624 / 414 / 362, 2048^2 264 / 259 / 230, 750^2 187 / 213 / 143, 512^2 133 / 145 / 102;
+//   one background pixel, 4-connectivity (a chain of tiles): 1001 x 1003 1184 / 1537 / 1061, 512^2
+//   630 / 824 / 553, 4096 x 202 1938 / 2559 / 1822.
 #include <cuda_runtime.h>
 
 #include <cstdint>
@@ -37,14 +43,6 @@ __device__ __forceinline__ uint32_t site_d2(int y, int x, uint32_t s) {
     const uint32_t dy = (uint32_t)(y - (int)(s >> 16)), dx = (uint32_t)(x - (int)(s & 0xFFFFu));
     return s == kNoSite ? 0xFFFFFFFFu : dy * dy + dx * dx;
 }
-// Keep (best, bd) or take cand if it is strictly closer to (y, x).
-__device__ __forceinline__ void offer(int y, int x, uint32_t cand, uint32_t &best, uint32_t &bd) {
-    const uint32_t d = site_d2(y, x, cand);
-    const bool take = d < bd;
-    best = take ? cand : best;
-    bd = take ? d : bd;
-}
-
 // A warp's tile with its one-pixel halo: row y0 + r at index r + 1, column x0 + c at c + 1. The pair
 // of columns 2c - 1, 2c of a row is 8-byte aligned: lane c reads its two pixels and
 // both their horizontal neighbours in two 64-bit accesses.
@@ -70,25 +68,31 @@ struct EdtWork {
 constexpr uint32_t kRowBits = (1u << ETH) - 1u;
 
 // Loads the tile and its halo; returns the rows that hold a foreground pixel (only those can
-// change: a background pixel is its own site).
+// change: a background pixel is its own site). In two halves: all 36 loads of a lane at once do not
+// fit 64 registers (80 bytes of spills against 40; one background pixel in 512^2 266 us against 248).
 __device__ uint32_t edt_load(const ImageView &im, EdtSmem &t, int y0, int x0, int lane) {
     uint32_t fg = 0;
-    uint32_t v0[ETH + 2], v1[ETH + 2];
-#pragma unroll
-    for (int r = 0; r < ETH + 2; r++) {
-        v0[r] = ld_site(im, y0 + r - 1, x0 + lane);
-        v1[r] = ld_site(im, y0 + r - 1, x0 + 32 + lane);
-    }
     const uint32_t hl = ld_site(im, y0 + lane - 1, x0 - 1), hr = ld_site(im, y0 + lane - 1, x0 + ETW);
 #pragma unroll
-    for (int r = 0; r < ETH + 2; r++) {
-        t.s[r][lane + 1] = v0[r];
-        t.s[r][lane + 33] = v1[r];
-        if (r >= 1 && r <= ETH) {
-            const int y = y0 + r - 1;
-            const uint32_t self = ((uint32_t)y << 16) | (uint32_t)(x0 + lane);
-            const bool f = y < im.H && ((x0 + lane < im.W && v0[r] != self) || (x0 + 32 + lane < im.W && v1[r] != self + 32u));
-            if (__any_sync(0xffffffffu, f)) fg |= 1u << (r - 1);
+    for (int h = 0; h < 2; h++) {
+        constexpr int N = (ETH + 2) / 2;
+        uint32_t v0[N], v1[N];
+#pragma unroll
+        for (int k = 0; k < N; k++) {
+            v0[k] = ld_site(im, y0 + h * N + k - 1, x0 + lane);
+            v1[k] = ld_site(im, y0 + h * N + k - 1, x0 + 32 + lane);
+        }
+#pragma unroll
+        for (int k = 0; k < N; k++) {
+            const int r = h * N + k;
+            t.s[r][lane + 1] = v0[k];
+            t.s[r][lane + 33] = v1[k];
+            if (r >= 1 && r <= ETH) {
+                const int y = y0 + r - 1;
+                const uint32_t self = ((uint32_t)y << 16) | (uint32_t)(x0 + lane);
+                const bool f = y < im.H && ((x0 + lane < im.W && v0[k] != self) || (x0 + 32 + lane < im.W && v1[k] != self + 32u));
+                fg |= (uint32_t)f << (r - 1);
+            }
         }
     }
     if (lane < ETH + 2) {
@@ -96,7 +100,7 @@ __device__ uint32_t edt_load(const ImageView &im, EdtSmem &t, int y0, int x0, in
         t.s[lane][ETW + 1] = hr;
     }
     __syncwarp();
-    return fg;
+    return __reduce_or_sync(0xffffffffu, fg);
 }
 
 // The halo again; adds the rows that its changes may change to the work.
@@ -124,44 +128,108 @@ __device__ void edt_reload_halo(const ImageView &im, EdtSmem &t, int y0, int x0,
     __syncwarp();
 }
 
-// One row from its own sites and the previous row of the pass (DIR +1: the row above). Returns
-// whether a pixel changed (warp-uniform).
+__device__ __forceinline__ void ld4(const uint32_t *p, uint32_t (&q)[4]) {
+    const uint2 a = *reinterpret_cast<const uint2 *>(p), b = *reinterpret_cast<const uint2 *>(p + 2);
+    q[0] = a.x; q[1] = a.y; q[2] = b.x; q[3] = b.y;
+}
+// Squared distances of site s to (y, x) and (y, x + 1): (dx + 1)^2 = dx^2 + 2 dx + 1.
+__device__ __forceinline__ void site_d2_pair(int y, int x, uint32_t s, uint32_t &d0, uint32_t &d1) {
+    const uint32_t dy = (uint32_t)(y - (int)(s >> 16)), dx = (uint32_t)(x - (int)(s & 0xFFFFu)), d = dy * dy + dx * dx;
+    d0 = s == kNoSite ? 0xFFFFFFFFu : d;
+    d1 = s == kNoSite ? 0xFFFFFFFFu : d + 2u * dx + 1u;
+}
+// The first of three sites at the smallest of their distances, and that distance.
+__device__ __forceinline__ void nearest3(uint32_t s0, uint32_t s1, uint32_t s2, uint32_t d0, uint32_t d1, uint32_t d2,
+                                         uint32_t &s, uint32_t &d) {
+    d = __vimin3_u32(d0, d1, d2);
+    s = d0 == d ? s0 : (d1 == d ? s1 : s2);
+}
+
+// A row step: the pixels at columns xe and xe + 1 (sites q[1], q[2]) from their row's sites q and the
+// previous row's p, both of columns xe - 1 .. xe + 2. Own sites stay unless another is strictly
+// closer. What waits longest, the previous row's sites and then the even pixel's new one, is weighed
+// last: 3-way minima of distances and their sites, instead of ten offers one after the other.
 template <int CONN>
-__device__ __forceinline__ bool edt_row(EdtSmem &t, int r, int dir, int y, int xe, bool ve, bool vo, int lane) {
-    const int xo = xe + 1;
-    uint32_t *row = &t.s[r + 1][2 * lane];
-    const uint32_t *prv = &t.s[r + 1 - dir][2 * lane];
-    const uint2 a = *reinterpret_cast<const uint2 *>(row), b = *reinterpret_cast<const uint2 *>(row + 2);
-    const uint2 pa = *reinterpret_cast<const uint2 *>(prv), pb = *reinterpret_cast<const uint2 *>(prv + 2);
-    // even pixel: own, W, E, and the previous row's N (+ NW, NE)
-    uint32_t be_ = a.y, de = site_d2(y, xe, be_);
-    offer(y, xe, a.x, be_, de);
-    offer(y, xe, b.x, be_, de);
-    offer(y, xe, pa.y, be_, de);
+__device__ __forceinline__ bool edt_step(const uint32_t (&q)[4], const uint32_t (&p)[4], int y, int xe, bool ve, bool vo,
+                                         uint32_t &e, uint32_t &o) {
+    uint32_t dq2, eq2, dp1, ep1, dp2, ep2;   // d..: to the even pixel, e..: to the odd one
+    site_d2_pair(y, xe, q[2], dq2, eq2);
+    site_d2_pair(y, xe, p[1], dp1, ep1);
+    site_d2_pair(y, xe, p[2], dp2, ep2);
+    uint32_t sv, dv, su, du, t, dt;
+    nearest3(q[1], q[0], q[2], site_d2(y, xe, q[1]), site_d2(y, xe, q[0]), dq2, sv, dv);
+    const uint32_t eq3 = site_d2(y, xe + 1, q[3]);
     if (CONN == 8) {
-        offer(y, xe, pa.x, be_, de);
-        offer(y, xe, pb.x, be_, de);
+        nearest3(p[1], p[0], p[2], dp1, site_d2(y, xe, p[0]), dp2, t, dt);
+        sv = dt < dv ? t : sv;
+        const uint32_t ep3 = site_d2(y, xe + 1, p[3]);
+        nearest3(p[2], p[1], p[3], ep2, ep1, ep3, su, du);
+        su = eq3 <= du ? q[3] : su;
+        du = min(eq3, du);
+    } else {
+        sv = dp1 < dv ? p[1] : sv;
+        su = eq3 <= ep2 ? q[3] : p[2];
+        du = min(eq3, ep2);
     }
-    if (!ve) be_ = kNoSite;
-    // odd pixel: own, W (the even pixel, just updated), E, and the previous row
-    uint32_t bo_ = b.x, dd = site_d2(y, xo, bo_);
-    offer(y, xo, be_, bo_, dd);
-    offer(y, xo, b.y, bo_, dd);
-    offer(y, xo, pb.x, bo_, dd);
-    if (CONN == 8) {
-        offer(y, xo, pa.y, bo_, dd);
-        offer(y, xo, pb.y, bo_, dd);
+    e = ve ? sv : kNoSite;
+    // (of equally near sites the own one, then the even pixel's, then the others)
+    const uint32_t de = site_d2(y, xe + 1, e);
+    o = eq2 <= de && eq2 <= du ? q[2] : (de <= du ? e : su);
+    if (!vo) o = kNoSite;
+    return e != q[1] || o != q[2];
+}
+
+// One pass over the rows with work, in the order DIR (+1 down, -1 up). Rows that follow one another are
+// a run: the next row's sites are loaded ahead and the previous one's stay in registers (its
+// neighbour columns by shuffles beside the vote), so that a row does not wait for the one before to
+// pass through shared memory. Adds the rows that changed to `rows`.
+template <int CONN, int DIR>
+__device__ __forceinline__ void edt_pass(EdtSmem &t, EdtWork &w, uint32_t fg, int y0, int xe, bool ve, bool vo,
+                                         uint32_t &rows, int lane) {
+    uint32_t &v = DIR > 0 ? w.n : w.s, &u = DIR > 0 ? w.s : w.n;
+    for (uint32_t left = kRowBits;;) {
+        const uint32_t m = (v | w.h) & fg & left;
+        if (m == 0) break;
+        int r = DIR > 0 ? __ffs(m) - 1 : 31 - __clz(m);
+        uint32_t bit = 1u << r, q[4], p[4];
+        __syncwarp();   // rows written before are read by other lanes
+        ld4(&t.s[r + 1][2 * lane], q);
+        ld4(&t.s[r + 1 - DIR][2 * lane], p);
+        for (;;) {
+            uint32_t *row = &t.s[r + 1][2 * lane], nx[4], e, o;
+            ld4(&t.s[r + 1 + DIR][2 * lane], nx);
+            const bool ch = edt_step<CONN>(q, p, y0 + r, xe, ve, vo, e, o);
+            if (CONN == 8) {
+                p[0] = __shfl_up_sync(0xffffffffu, o, 1);
+                p[3] = __shfl_down_sync(0xffffffffu, e, 1);
+                if (lane == 0) p[0] = q[0];
+                if (lane == 31) p[3] = q[3];
+            }
+            p[1] = e;
+            p[2] = o;
+            const bool any = __any_sync(0xffffffffu, ch);
+            __syncwarp();   // every lane has read the row
+            if (ch) {
+                row[1] = e;
+                row[2] = o;
+            }
+            const uint32_t next = DIR > 0 ? bit << 1 : bit >> 1, prev = DIR > 0 ? bit >> 1 : bit << 1;
+            v &= ~bit;
+            w.h &= ~bit;
+            if (any) {
+                rows |= bit;
+                w.h |= bit;
+                v |= next;
+                u |= prev;
+            }
+            left = DIR > 0 ? ~(next - 1u) : bit - 1u;
+            if (((v | w.h) & fg & next) == 0) break;   // (fg holds rows of the tile only)
+            r += DIR;
+            bit = next;
+#pragma unroll
+            for (int i = 0; i < 4; i++) q[i] = nx[i];
+        }
     }
-    if (!vo) bo_ = kNoSite;
-    const bool ch = be_ != a.y || bo_ != b.x;
-    const bool any = __any_sync(0xffffffffu, ch);
-    __syncwarp();   // every lane has read the row
-    if (ch) {
-        row[1] = be_;
-        row[2] = bo_;
-    }
-    __syncwarp();
-    return any;
 }
 
 // Passes until the tile is settled; returns the rows that changed. Rows are taken in the order
@@ -172,38 +240,11 @@ __device__ uint32_t edt_settle(EdtSmem &t, EdtWork &w, uint32_t fg, int y0, int 
     const bool ve = xe < W, vo = xe + 1 < W;
     uint32_t rows = 0;
     while ((w.n | w.s | w.h) & fg) {
-        for (uint32_t left = kRowBits;;) {   // down
-            const uint32_t m = (w.n | w.h) & fg & left;
-            if (m == 0) break;
-            const int r = __ffs(m) - 1;
-            const uint32_t bit = 1u << r;
-            left = ~((bit << 1) - 1u);
-            w.n &= ~bit;
-            w.h &= ~bit;
-            if (edt_row<CONN>(t, r, 1, y0 + r, xe, ve, vo, lane)) {
-                rows |= bit;
-                w.h |= bit;
-                w.n |= bit << 1;
-                w.s |= bit >> 1;
-            }
-        }
-        for (uint32_t left = kRowBits;;) {   // up
-            const uint32_t m = (w.s | w.h) & fg & left;
-            if (m == 0) break;
-            const int r = 31 - __clz(m);
-            const uint32_t bit = 1u << r;
-            left = bit - 1u;
-            w.s &= ~bit;
-            w.h &= ~bit;
-            if (edt_row<CONN>(t, r, -1, y0 + r, xe, ve, vo, lane)) {
-                rows |= bit;
-                w.h |= bit;
-                w.n |= bit << 1;
-                w.s |= bit >> 1;
-            }
-        }
+        edt_pass<CONN, 1>(t, w, fg, y0, xe, ve, vo, rows, lane);
+        edt_pass<CONN, -1>(t, w, fg, y0, xe, ve, vo, rows, lane);
         passes += 2;
     }
+    __syncwarp();
     return rows;
 }
 
@@ -257,16 +298,17 @@ __device__ uint32_t edt_notify_mask(const EdtSmem &t, int y0, int x0, int lane) 
 // Stores the changed rows' sites and, when asked for (D), their squared distances.
 __device__ void edt_store(const ImageView &im, uint32_t *D, const EdtSmem &t, int y0, int x0, uint32_t rows, int lane) {
     uint32_t *S = reinterpret_cast<uint32_t *>(im.J);
-    for (uint32_t m = rows; m; m &= m - 1) {
-        const int r = __ffs(m) - 1;
-        const size_t row = (size_t)(y0 + r) * im.W;
-#pragma unroll
-        for (int q = 0; q < 2; q++) {
-            const int x = x0 + lane + 32 * q;
-            if (x >= im.W) continue;
-            const uint32_t v = t.s[r + 1][lane + 1 + 32 * q];
-            __stcg(S + row + x, v);
-            if (D) __stcg(D + row + x, site_d2(y0 + r, x, v));
+    const bool in0 = x0 + lane < im.W, in1 = x0 + 32 + lane < im.W;
+#pragma unroll 4
+    for (int r = 0; r < ETH; r++) {
+        if (!((rows >> r) & 1u)) continue;   // (changed rows lie inside the image)
+        const size_t e = (size_t)(y0 + r) * im.W + x0 + lane;
+        const uint32_t v0 = t.s[r + 1][lane + 1], v1 = t.s[r + 1][lane + 33];
+        if (in0) __stcg(S + e, v0);
+        if (in1) __stcg(S + e + 32, v1);
+        if (D) {
+            if (in0) __stcg(D + e, site_d2(y0 + r, x0 + lane, v0));
+            if (in1) __stcg(D + e + 32, site_d2(y0 + r, x0 + 32 + lane, v1));
         }
     }
 }

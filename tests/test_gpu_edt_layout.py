@@ -1,6 +1,6 @@
 """GPU: the distance transform's row skipping and its four-pixel initialisation at the edges:
 widths on both sides of a multiple of 4 and of the 64-column tile, arrays that are not aligned for
-the wide accesses, rows without foreground between rows with it."""
+the wide accesses, rows without foreground between rows with it, runs of rows."""
 import numpy as np
 import pytest
 
@@ -34,3 +34,17 @@ def test_layouts(W, conn):
             s2 = site2.cpu().numpy().view(np.uint32).astype(np.int64)
             yy, xx = np.mgrid[0:H, 0:W]
             check_valid(fg, s2 >> 16, s2 & 0xFFFF, (yy - (s2 >> 16)) ** 2 + (xx - (s2 & 0xFFFF)) ** 2, conn)
+
+
+@pytest.mark.parametrize("H,W", [(1, 4000), (4000, 1), (700, 66), (66, 700), (333, 335)])
+@pytest.mark.parametrize("conn", [4, 8])
+def test_one_site_travels_through_every_tile(H, W, conn):
+    # rows of a tile that follow one another are one run, from above and from below; one site is exact
+    for y, x in ((0, 0), (H - 1, W - 1), (H // 2, W // 2)):
+        fg = np.ones((H, W), np.uint8)
+        fg[y, x] = 0
+        d2 = torch.empty((H, W), dtype=torch.int32, device="cuda")
+        T = iwpp.DistanceTransform(H, W)
+        assert T(torch.from_numpy(fg).cuda(), torch.empty_like(d2), d2, conn) == 0 and T.status() == 0
+        yy, xx = np.mgrid[0:H, 0:W]
+        assert np.array_equal(d2.cpu().numpy(), (yy - y) ** 2 + (xx - x) ** 2)
