@@ -564,7 +564,8 @@ IWPP_API int iwpp_skiz(const uint32_t *markers, const uint8_t *mask, uint32_t *z
  *   site_out     device, H x W uint32 (4-byte aligned): the site of each pixel packed
  *                as (y << 16) | x, 0xFFFFFFFF where no background exists
  *   dist2_out    device, H x W uint32 or NULL: squared distance to the site
- *                (0xFFFFFFFF where there is none)
+ *                (0xFFFFFFFF where there is none); may be site_out itself, and may
+ *                contain the mask: it is then written last
  *   H, W         1 .. 32767 (squared distances then fit in 32 bits)
  *   connectivity 4 or 8 (the neighbourhood the sites travel through)
  *   workspace    device, 256-byte aligned, iwpp_edt_workspace_bytes(H, W) bytes

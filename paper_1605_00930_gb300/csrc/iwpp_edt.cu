@@ -418,6 +418,12 @@ __global__ void __launch_bounds__(kThreads, 8) edt_drain_kernel(EngineArgs a, ui
     flush_stats(a, st, idle, busy, lane);
 }
 
+// The distances by themselves, from the final sites (which they may overwrite).
+__global__ void edt_dist2_kernel(const uint32_t *S, uint32_t *D, int W, size_t n) {
+    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
+        D[i] = site_d2((int)(i / W), (int)(i % W), S[i]);
+}
+
 // Workspace: header (256 B) | tile states | tile-queue ring.
 struct EdtLayout {
     size_t state, queue, total;
@@ -472,13 +478,21 @@ extern "C" int iwpp_edt(const void *mask, uint32_t *site_out, uint32_t *dist2_ou
     if (cudaMemsetAsync(base, 0, L.queue + (size_t)L.ntiles * 4, s) != cudaSuccess) return IWPP_ERR_CUDA;
     const int sms = device_sm_count();
     if (sms <= 0) return IWPP_ERR_CUDA;
+    // Distances that go where the sites or the mask are cannot be written with the sites: they follow
+    // the drain (41 us at 4096^2).
+    const size_t n = (size_t)H * (size_t)W;
+    const auto shares = [&](const void *p, size_t bytes) {
+        const uintptr_t d = (uintptr_t)dist2_out, q = (uintptr_t)p;
+        return d < q + bytes && q < d + 4 * n;
+    };
+    uint32_t *const D = dist2_out && (shares(site_out, 4 * n) || shares(mask, n)) ? nullptr : dist2_out;
     const uint32_t warps_needed = L.ntiles;
     uint32_t ig = (warps_needed + 7) / 8;
     if (ig > (uint32_t)sms * 8) ig = (uint32_t)sms * 8;
     const bool vec = (W & 3) == 0 && ((uintptr_t)mask & 3) == 0 && ((uintptr_t)site_out & 15) == 0 &&
-                     ((uintptr_t)dist2_out & 15) == 0;
-    if (vec) edt_init_kernel<true><<<ig, 256, 0, s>>>(a, dist2_out);
-    else edt_init_kernel<false><<<ig, 256, 0, s>>>(a, dist2_out);
+                     ((uintptr_t)D & 15) == 0;
+    if (vec) edt_init_kernel<true><<<ig, 256, 0, s>>>(a, D);
+    else edt_init_kernel<false><<<ig, 256, 0, s>>>(a, D);
     const size_t smem = kEdtSmemPerWarp * kWarpsPerCta;
     void (*drain)(EngineArgs, uint32_t *) = connectivity == 8 ? edt_drain_kernel<8> : edt_drain_kernel<4>;
     int bps = 0;
@@ -487,6 +501,7 @@ extern "C" int iwpp_edt(const void *mask, uint32_t *site_out, uint32_t *dist2_ou
     long long g = (long long)bps * sms;
     const long long need = ((long long)L.ntiles + kWarpsPerCta - 1) / kWarpsPerCta;
     if (g > need) g = need;
-    drain<<<(int)g, kThreads, smem, s>>>(a, dist2_out);
+    drain<<<(int)g, kThreads, smem, s>>>(a, D);
+    if (D != dist2_out) edt_dist2_kernel<<<sms * 8, 256, 0, s>>>(site_out, dist2_out, (int)W, n);
     return cudaGetLastError() == cudaSuccess ? IWPP_OK : IWPP_ERR_CUDA;
 }

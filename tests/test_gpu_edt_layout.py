@@ -48,3 +48,21 @@ def test_one_site_travels_through_every_tile(H, W, conn):
         assert T(torch.from_numpy(fg).cuda(), torch.empty_like(d2), d2, conn) == 0 and T.status() == 0
         yy, xx = np.mgrid[0:H, 0:W]
         assert np.array_equal(d2.cpu().numpy(), (yy - y) ** 2 + (xx - x) ** 2)
+
+
+@pytest.mark.parametrize("H,W", [(1, 1), (16, 64), (37, 201), (200, 333)])
+def test_distances_over_the_sites_or_the_mask(H, W):
+    fg = np.ones((H, W), np.uint8)
+    fg[H // 2, W // 3] = 0
+    yy, xx = np.mgrid[0:H, 0:W]
+    want = (yy - H // 2) ** 2 + (xx - W // 3) ** 2   # one site: exact
+    T = iwpp.DistanceTransform(H, W)
+    out = torch.empty((H, W), dtype=torch.int32, device="cuda")
+    assert T(torch.from_numpy(fg).cuda(), out, out, 8) == 0 and T.status() == 0
+    assert np.array_equal(out.cpu().numpy(), want)
+    mask = out.view(torch.uint8).reshape(-1)[:H * W].view(H, W)   # the mask where the distances go
+    mask.copy_(torch.from_numpy(fg))
+    site = torch.empty_like(out)
+    assert T(mask, site, out, 8) == 0 and T.status() == 0
+    assert np.array_equal(out.cpu().numpy(), want)
+    assert np.all(site.cpu().numpy() == ((H // 2) << 16 | (W // 3)))
