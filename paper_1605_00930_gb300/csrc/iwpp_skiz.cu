@@ -14,9 +14,9 @@
 // its tile for a visit.
 //
 // A row step weighs ~70 instructions (10 candidates of two words each per lane); what bounds the
-// drain is the number of row steps and the warps there are to overlap them.
-// 4096^2 porous domain, 8-connectivity, zones, distances and label pairs: 3.29 ms with the tile
-// in registers (152 of them, 12 warps per SM, every row in every pass), 1.2 ms now.
+// drain is the number of row steps, the latency of one and the warps there are to overlap them.
+// 4096^2 porous domain, 2000 markers, 8-connectivity, zones, distances and label pairs, whole call:
+// 3.31 ms with the tile in registers (152 of them, 12 warps per SM, every row in every pass), 1.19 ms now.
 #include <cuda_runtime.h>
 
 #include <cstdint>
@@ -70,7 +70,9 @@ __device__ __forceinline__ void join(const unsigned long long (&q)[N], uint32_t 
 struct SkOp {
     using Px = unsigned long long;   // (d << 32) | l
     struct Aux {};
+    struct RowAux {};
     struct Ctx {};
+    static __device__ __forceinline__ RowAux row_aux(const Aux &, int, int) { return RowAux{}; }
     static __device__ __forceinline__ Px none() { return pack(St{kBlocked, kNoLab}); }
     static __device__ __forceinline__ Px load(const ImageView &im, size_t e) {
         return __ldcg(reinterpret_cast<const Px *>(im.J) + e);
@@ -82,8 +84,7 @@ struct SkOp {
     static __device__ __forceinline__ uint32_t halo_aux(const Aux &, int, int) { return 0; }
 
     template <int CONN>
-    static __device__ __forceinline__ bool row(const Px (&q)[4], const Px (&p)[4], const Aux &, const Ctx &, int, int,
-                                               Px &e, Px &o) {
+    static __device__ __forceinline__ bool row(const Px (&q)[4], const Px (&p)[4], const RowAux &, int, Px &e, Px &o) {
         uint32_t m, lc;
         if (CONN == 8) {
             const Px c[5] = {q[0], q[2], p[0], p[1], p[2]};
@@ -153,7 +154,7 @@ __global__ void __launch_bounds__(256) sk_init_kernel(EngineArgs a, const uint32
 }
 
 #ifndef IWPP_SKIZ_MINB
-#define IWPP_SKIZ_MINB 4   // CTAs (of 8 warps) per SM: 64 registers; 3 are 9 % slower on 4096^2
+#define IWPP_SKIZ_MINB 4   // CTAs (of 8 warps) per SM: 64 registers; 3 were 9 % slower on 4096^2 before rows became runs
 #endif
 template <int CONN>
 __global__ void __launch_bounds__(kSmThreads, IWPP_SKIZ_MINB) sk_drain_kernel(EngineArgs a) {

@@ -12,11 +12,17 @@
 // bottom) settles n, an up pass s, either h when it changes nothing. A tile that was visited
 // before starts with the rows next to its halo that the halo can change, and nothing else.
 //
-// Strips exchange after one pass pair, eight strips of 8 rows. Whole calls of the drains with
-// (warps, exchange): watershed of 2048^2 u16 and 4096^2 u16, influence zones of 4096^2 and 1000^2:
+// Strips exchange after one pass pair, eight strips of 8 rows. Both were chosen with rows that each
+// went through shared memory (and plain accesses between strips), calls with (warps, exchange):
+// watershed of 2048^2 u16 and 4096^2 u16, influence zones of 4096^2 and 1000^2:
 // (4, when clean) 1565 / 2742 / 1173 / 642 us, (4, pair) 1282 / 2489 / 1133 / 527, (8, when clean)
 // 1500 / 3119 / 1316 / 591, (8, pair) 1122 / 2946 / 1171 / 423, (8, single pass) 1432 / 2974 / 1217 / 458,
-// (16, pair) 1324 / 4011 / 1767 / 440. Against one warp's 16 rows in registers: 1541 / 4565 / 3252 / 1135.
+// (16, pair) 1324 / 4011 / 1767 / 440. They have not been timed again since.
+//
+// Runs of rows (sm_pass_pair), whole calls, against strips of 16 rows in one warp's registers (the form
+// before these tiles), 57 watersheds and 57 influence zones from 200^2 to 4096^2, u8 and u16, both
+// connectivities: geometric mean 1.63 and 2.58 times as fast, the slowest 1.16 and 2.17 (each
+// row through shared memory: 1.04 and 2.05, with 200^2 watersheds down to 0.88).
 //
 // Strips read the adjacent strips' boundary rows where they lie. A pixel is written by its own strip
 // only; between two barriers those writes, and the reads of another strip's row, are single relaxed
@@ -25,7 +31,7 @@
 // valid; the strip whose row changed hands its neighbour the row again at the next barrier.
 //
 // Op: the operator. Px (a pixel's state, one aligned 4- or 8-byte word), Aux (what it needs
-// beside it) and Ctx (kernel arguments), none() (outside the image), load / store, load_aux,
+// beside it), RowAux (a lane's part of that for a row, row_aux) and Ctx (kernel arguments), none() (outside the image), load / store, load_aux,
 // row<CONN> (one lane's two pixels of a row step, from columns 2c - 1 .. 2c + 2 of the row and of the
 // one before it), halo_aux and changes (whether pixels offered to a halo pixel change it).
 #pragma once
@@ -163,25 +169,26 @@ __device__ RowWork sm_revisit_work(const SmemTile<Op> &S, const typename Op::Ctx
     return k;
 }
 
-// One down and one up pass over the strip's rows with work; returns the rows changed.
+// One down and one up pass over the strip's rows with work; returns the rows changed. Rows that
+// follow one another are a run: the next row is loaded ahead and the previous one stays in registers (its
+// neighbour columns by shuffles beside the vote), so that a row does not wait for the one before
+// to pass through shared memory.
 template <class Op, int CONN>
 __device__ uint32_t sm_pass_pair(SmemTile<Op> &S, const typename Op::Ctx &ctx, RowWork &k, uint32_t &passes, int w, int lane) {
+    using Px = typename Op::Px;
     uint32_t rows = 0;
-#pragma unroll 1
+#pragma unroll   // (a direction known at compile time: 5-12 % faster)
     for (int dir = 1; dir >= -1; dir -= 2) {
-        uint32_t &v = dir > 0 ? k.n : k.s;
+        uint32_t v = dir > 0 ? k.n : k.s, u = dir > 0 ? k.s : k.n;
         for (uint32_t left = kSmRows;;) {
             const uint32_t m = (v | k.h) & left;
             if (m == 0) break;
-            const int r = dir > 0 ? __ffs(m) - 1 : 31 - __clz(m);
-            const uint32_t bit = 1u << r;
-            left = dir > 0 ? ~((bit << 1) - 1u) & kSmRows : bit - 1u;
-            v &= ~bit;
-            k.h &= ~bit;
-            const int ri = kSmStrip * w + r + 1;
-            typename Op::Px *row = &S.v[ri][2 * lane];
-            const typename Op::Px *prv = &S.v[ri - dir][2 * lane];
-            typename Op::Px q[4], p[4], e, o;
+            int r = dir > 0 ? __ffs(m) - 1 : 31 - __clz(m);
+            uint32_t bit = 1u << r;
+            Px q[4], p[4];
+            __syncwarp();   // rows written before are read by other lanes
+            Px *row = &S.v[kSmStrip * w + r + 1][2 * lane];
+            const Px *prv = row - dir * kSmPitch;
             sm_ld4(row, q);
             if (dir > 0 ? r == 0 && w > 0 : r == kSmStrip - 1 && w < kSmWarps - 1) {   // another strip's row
 #pragma unroll
@@ -189,22 +196,50 @@ __device__ uint32_t sm_pass_pair(SmemTile<Op> &S, const typename Op::Ctx &ctx, R
             } else {
                 sm_ld4(prv, p);
             }
-            const bool ch = Op::template row<CONN>(q, p, S.aux, ctx, ri - 1, lane, e, o);
-            const bool any = __any_sync(0xffffffffu, ch);
-            __syncwarp();   // every lane has read the row
-            if (ch) {
-                sm_st_relaxed(row + 1, e);
-                sm_st_relaxed(row + 2, o);
-            }
-            __syncwarp();
-            if (any) {
-                rows |= bit;
-                k.h |= bit;
-                k.n |= (bit << 1) & kSmRows;
-                k.s |= bit >> 1;
+            typename Op::RowAux x = Op::row_aux(S.aux, kSmStrip * w + r, lane);
+            for (;;) {
+                const uint32_t next = dir > 0 ? (bit << 1) & kSmRows : bit >> 1;
+                const int step = next ? dir : 0;   // (at the strip's end the row itself again)
+                Px nx[4], e, o;
+                sm_ld4(row + step * kSmPitch, nx);
+                const typename Op::RowAux xn = Op::row_aux(S.aux, kSmStrip * w + r + step, lane);
+                const bool ch = Op::template row<CONN>(q, p, x, lane, e, o);
+                if (CONN == 8) {
+                    p[0] = __shfl_up_sync(0xffffffffu, o, 1);
+                    p[3] = __shfl_down_sync(0xffffffffu, e, 1);
+                    if (lane == 0) p[0] = q[0];
+                    if (lane == 31) p[3] = q[3];
+                }
+                p[1] = e;
+                p[2] = o;
+                const bool any = __any_sync(0xffffffffu, ch);
+                __syncwarp();   // every lane has read the row
+                if (ch) {
+                    sm_st_relaxed(row + 1, e);
+                    sm_st_relaxed(row + 2, o);
+                }
+                v &= ~bit;
+                k.h &= ~bit;
+                if (any) {
+                    rows |= bit;
+                    k.h |= bit;
+                    v |= next;
+                    u |= dir > 0 ? bit >> 1 : (bit << 1) & kSmRows;
+                }
+                left = dir > 0 ? ~((bit << 1) - 1u) & kSmRows : bit - 1u;
+                if (((v | k.h) & next) == 0) break;
+                r += dir;
+                bit = next;
+                row += dir * kSmPitch;
+                x = xn;
+#pragma unroll
+                for (int i = 0; i < 4; i++) q[i] = nx[i];
             }
         }
+        k.n = dir > 0 ? v : u;
+        k.s = dir > 0 ? u : v;
     }
+    __syncwarp();
     passes += 2;
     return rows;
 }

@@ -11,9 +11,10 @@
 // reach a pixel at its level depends on the order of work, as in any flooding watershed.
 //
 // A row step weighs ~60 instructions (10 offers of three per lane); what bounds the drain is the
-// number of row steps and the warps there are to overlap them. 2048^2 u16 gradient, 500 markers,
-// 8-connectivity: 1.54 ms with the tile in registers (254 of them, 8 warps per SM, every row in
-// every pass), 1.12 ms now; 4096^2 with 2000 markers 4.57 and 2.95.
+// number of row steps, the latency of one and the warps there are to overlap them. Whole calls with levels,
+// 8-connectivity, tiles of one warp's registers (254 of them, 8 warps per SM, every row in every pass)
+// and now: 2048^2 u16 gradient, 500 markers 1.65 and 1.12 ms, 4096^2 u16, a marker per 4000 pixels
+// 4.50 and 2.96, 200^2 u8, two markers 0.230 and 0.197.
 #include <cuda_runtime.h>
 
 #include <cstdint>
@@ -57,7 +58,13 @@ struct WsOp {
         uint32_t fixed[kSmSide][2];          // per row: lanes whose even / odd pixel is fixed (a marker, or outside)
         uint32_t hg[4][kSmSide + 2];         // the halo's gradient << 16 per side (all ones outside the image)
     };
+    struct RowAux {
+        uint32_t g, fe, fo;   // the lane's gradient pair; which lanes' pixels are fixed
+    };
     using Ctx = WsArgs;
+    static __device__ __forceinline__ RowAux row_aux(const Aux &x, int r, int lane) {
+        return RowAux{x.g[r][lane], x.fixed[r][0], x.fixed[r][1]};
+    }
     static __device__ __forceinline__ Px none() { return kUnreached; }
     static __device__ __forceinline__ Px load(const ImageView &im, size_t e) {
         return __ldcg(reinterpret_cast<const uint32_t *>(im.J) + e);
@@ -97,10 +104,9 @@ struct WsOp {
     }
 
     template <int CONN>
-    static __device__ __forceinline__ bool row(const Px (&q)[4], const Px (&p)[4], const Aux &x, const Ctx &, int r,
-                                               int lane, Px &e, Px &o) {
-        const uint32_t gp = x.g[r][lane], ge = gp << 16, go = gp & 0xFFFF0000u;
-        const uint32_t fe = x.fixed[r][0], fo = x.fixed[r][1];
+    static __device__ __forceinline__ bool row(const Px (&q)[4], const Px (&p)[4], const RowAux &x, int lane, Px &e,
+                                               Px &o) {
+        const uint32_t ge = x.g << 16, go = x.g & 0xFFFF0000u;
         // (the offers of this row first, those of the row just written last: the shorter chain)
         uint32_t v = __vimin3_u32(q[1], offer_ws(q[0], ge), offer_ws(q[2], ge));
         uint32_t u = __vimin3_u32(q[2], offer_ws(q[3], go), offer_ws(p[2], go));
@@ -110,8 +116,8 @@ struct WsOp {
         } else {
             v = min(v, offer_ws(p[1], ge));
         }
-        e = (fe >> lane) & 1u ? q[1] : v;
-        o = (fo >> lane) & 1u ? q[2] : min(u, offer_ws(e, go));
+        e = (x.fe >> lane) & 1u ? q[1] : v;
+        o = (x.fo >> lane) & 1u ? q[2] : min(u, offer_ws(e, go));
         return e != q[1] || o != q[2];
     }
     static __device__ __forceinline__ bool changes(Px h, uint32_t g16, const Px (&q)[3], int n) {
@@ -164,7 +170,7 @@ __global__ void __launch_bounds__(256) ws_init_kernel(EngineArgs a, WsArgs w, ui
 }
 
 #ifndef IWPP_WS_MINB
-#define IWPP_WS_MINB 3   // CTAs (of 8 warps) per SM: 80 registers; 4 (64) are 8 % faster on 4096^2, 10 % slower on 2048^2
+#define IWPP_WS_MINB 3   // CTAs (of 8 warps) per SM: 80 registers; 4 (64) were 8 % faster on 4096^2 and 10 % slower on 2048^2 before rows became runs
 #endif
 template <int CONN>
 __global__ void __launch_bounds__(kSmThreads, IWPP_WS_MINB) ws_drain_kernel(EngineArgs a, WsArgs wa) {

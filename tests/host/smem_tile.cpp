@@ -42,6 +42,14 @@ struct Px {
 };
 static Px sm_ld_relaxed(const Px *p) { note(p, false, true); return Px(p->v); }
 static void sm_st_relaxed(Px *p, const Px &v) { note(p, true, true); p->v = v.v; }
+static Px __shfl_up_sync(uint32_t, const Px &v, int n) {
+    const int l = H.cur % 32;
+    return Px(H.warp_meet(v.v)[l < n ? l : l - n]);
+}
+static Px __shfl_down_sync(uint32_t, const Px &v, int n) {
+    const int l = H.cur % 32;
+    return Px(H.warp_meet(v.v)[l + n > 31 ? l : l + n]);
+}
 static void sm_ld4(const Px *p, Px (&q)[4]) { for (int i = 0; i < 4; i++) q[i] = p[i]; }
 
 constexpr unsigned long long kFar = 1ull << 62, kWall = ~0ull, kStep = 1ull << 32;
@@ -51,14 +59,16 @@ static unsigned long long step(unsigned long long own, unsigned long long q) {
 struct TestOp {
     using Px = ::Px;
     struct Aux {};
+    struct RowAux {};
     struct Ctx {};
+    static RowAux row_aux(const Aux &, int, int) { return RowAux{}; }
     static Px none() { return Px(kWall); }
     static Px load(const ImageView &im, size_t e) { return Px(im.J[e]); }
     static void store(const ImageView &im, size_t e, const Px &v) { note(&v, false, false); im.J[e] = v.v; }
     static void load_aux(Aux &, const ImageView &, const Ctx &, int, int, int, int) {}
     static uint32_t halo_aux(const Aux &, int, int) { return 0; }
     template <int CONN>
-    static bool row(const Px (&q)[4], const Px (&p)[4], const Aux &, const Ctx &, int, int, Px &e, Px &o) {
+    static bool row(const Px (&q)[4], const Px (&p)[4], const RowAux &, int, Px &e, Px &o) {
         unsigned long long v = step(step(step(q[1].v, q[0].v), q[2].v), p[1].v), u = step(q[2].v, p[2].v);
         if (CONN == 8) {
             v = step(step(v, p[0].v), p[2].v);

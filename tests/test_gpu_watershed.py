@@ -60,6 +60,21 @@ def test_plateaus_and_ridges(iw):
         check_labels(markers, grad, lab, lev, 8)
 
 
+@pytest.mark.parametrize("is16,conn", [(False, 8), (True, 4)])
+def test_more_tiles_than_workers(iw, is16, conn):
+    # 1280 tiles wait for 456 workers and are visited again and again, by other workers
+    rng = np.random.default_rng([112, conn])
+    H, W = 2047, 2501
+    f = synth.blob_field_u8(H, W, 600, rng)
+    grad = synth.to_u16(f) if is16 else f
+    markers = np.zeros((H, W), np.uint32)
+    markers[rng.integers(0, H, 60), rng.integers(0, W, 60)] = rng.integers(1, 50, 60)
+    lab, lev = run(iw, markers, grad, conn)
+    _, olev = oracle.watershed(markers, grad, conn)
+    np.testing.assert_array_equal(lev, olev)
+    check_labels(markers, grad, lab, lev, conn, max_labels_checked=4)
+
+
 def test_bad_label_reported(iw):
     markers = np.zeros((40, 70), np.uint32)
     markers[3, 4] = 70000
