@@ -367,41 +367,44 @@ struct RegTile {
         return chg;
     }
 
-    // One down pass; returns this lane's mask of changed rows. For 8-connectivity the
-    // neighbourhood {W, E, N, NW, NE} of a row is the horizontal max of max(row, row above)
-    // (max commutes with the shift), so one shuffle pair per row serves both rows. For
-    // 4-connectivity each row first takes N (clamped to I: a valid update of every pixel) and then
-    // W / E from those new values, so a path that steps down and sideways advances within one pass
-    // (measured: 7 instead of 16 passes per visit on the 4096^2 tissue image). The side halo has
-    // been absorbed before (absorb_side): a row step is 6 arithmetic instructions (with
-    // 3-input maxima; 9 and a shared load when each step took the side halo in). They bound the
-    // drain: min/max.u16x2 and byte permutes issue every second cycle of a scheduler, shuffles every
-    // fourth (measured).
-    // Returns the mask of changed rows.
-    static __device__ __forceinline__ uint32_t pass_down(uint32_t (&J)[TH], const uint32_t (&I)[TH], uint32_t jt) {
-        uint32_t chg = 0, up = jt;
+    // One down pass of the register solver; returns this lane's mask of changed rows. For 8-connectivity
+    // the neighbourhood {W, E, N, NW, NE} of a row is the horizontal max of max(row, row above)
+    // (max commutes with the shift), so one shuffle pair per row serves both rows; the side halo is
+    // then the max of the two rows' halo words. For 4-connectivity each row first takes N (clamped
+    // to I: a valid update of every pixel) and then W / E from those new values, so a path that steps
+    // down and sideways advances within one pass (measured: 7 instead of 16 passes per visit on the
+    // 4096^2 tissue image); the side halo has been absorbed before. (Absorbing it for 8-connectivity
+    // too was no faster with these passes, and 1-2 % slower on fill-holes: 2048^2 2465 us against
+    // 2496, value levels at 512^2 291 against 298. 4-connectivity gains 2-4 %.)
+    static constexpr bool kAbsorb = CONN == 4;
+    static __device__ __forceinline__ uint32_t pass_down(const uint32_t *hx, uint32_t (&J)[TH], const uint32_t (&I)[TH],
+                                                         uint32_t jt, int lane) {
+        uint32_t chg = 0, up = jt, hprev = kAbsorb ? 0u : hx[0];
 #pragma unroll
         for (int r = 0; r < TH; r++) {
-            const uint32_t v = J[r];
-            const uint32_t nv = CONN == 8 ? min2(I[r], hmax_in(max2(v, up)))
+            const uint32_t hcur = kAbsorb ? 0u : hx[r + 1], v = J[r];
+            const uint32_t nv = CONN == 8 ? min2(I[r], hmax(max2(v, up), max2(hcur, hprev), lane))
                                           : min2(I[r], hmax_in(min2(I[r], max2(v, up))));
             chg |= (uint32_t)(nv != v) << r;
             J[r] = nv;
             up = nv;
+            hprev = hcur;
         }
         return chg;
     }
 
-    static __device__ __forceinline__ uint32_t pass_up(uint32_t (&J)[TH], const uint32_t (&I)[TH], uint32_t jb) {
-        uint32_t chg = 0, dn = jb;
+    static __device__ __forceinline__ uint32_t pass_up(const uint32_t *hx, uint32_t (&J)[TH], const uint32_t (&I)[TH],
+                                                       uint32_t jb, int lane) {
+        uint32_t chg = 0, dn = jb, hnext = kAbsorb ? 0u : hx[TH + 1];
 #pragma unroll
         for (int r = TH - 1; r >= 0; r--) {
-            const uint32_t v = J[r];
-            const uint32_t nv = CONN == 8 ? min2(I[r], hmax_in(max2(v, dn)))
+            const uint32_t hcur = kAbsorb ? 0u : hx[r + 1], v = J[r];
+            const uint32_t nv = CONN == 8 ? min2(I[r], hmax(max2(v, dn), max2(hcur, hnext), lane))
                                           : min2(I[r], hmax_in(min2(I[r], max2(v, dn))));
             chg |= (uint32_t)(nv != v) << r;
             J[r] = nv;
             dn = nv;
+            hnext = hcur;
         }
         return chg;
     }
@@ -410,7 +413,10 @@ struct RegTile {
     // chain depend on each other (two shuffles each), those of different chains do not. Rows at a
     // seam take the other chain's row as it was before the pass, on both sides of every seam
     // and in both directions, so that a pass that changes nothing after a pass in the other
-    // direction still leaves every pixel checked against all its neighbours. DIR +1: down, halo =
+    // direction still leaves every pixel checked against all its neighbours. The side halo has been
+    // absorbed before (absorb_side): a row step is 6 arithmetic instructions (with 3-input maxima; 9 and
+    // a shared load when each step took the side halo in). They bound the drain: min/max.u16x2 and byte
+    // permutes issue every second cycle of a scheduler, shuffles every fourth (measured). DIR +1: down, halo =
     // the row above the tile; -1: up, halo = the row below. Returns the sum of the lane's pixels
     // (value_sum): values never fall, so a pass changed a pixel exactly when the sum is another. The sum
     // is one dp2a per row, which issues beside the min / max / permute pipe that bounds a
@@ -792,14 +798,14 @@ __device__ void visit_tile_reg(const EngineArgs &a, const ImageView &im, uint32_
     IWPP_RT_MARK(0);
     uint32_t passes = 0;
     for (;;) {
-        uint32_t rows = RT::absorb_side(hx, J, I);
+        uint32_t rows = RT::kAbsorb ? RT::absorb_side(hx, J, I) : 0u;
         for (;;) {
 #if IWPP_REG_SWEEPS
             uint32_t ch = RT::sweep_raster(hx, J, I, jt, lane);
             ch |= RT::sweep_antiraster(hx, J, I, jb, lane);
 #else
-            uint32_t ch = RT::pass_down(J, I, jt);
-            ch |= RT::pass_up(J, I, jb);
+            uint32_t ch = RT::pass_down(hx, J, I, jt, lane);
+            ch |= RT::pass_up(hx, J, I, jb, lane);
 #endif
             passes += 2;
             rows |= ch;
