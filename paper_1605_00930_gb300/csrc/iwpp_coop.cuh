@@ -34,28 +34,14 @@ struct CoopShared {
 // 4096^2 u8 549 -> 516, 3001 x 2777 4-conn 373 -> 347, 4096^2 u16 fill-holes 2515 -> 2223,
 // 16384^2 seeds 9703 -> 9450, 48 uneven images 3477 -> 3346, 256 learned 12680 -> 12608; four
 // chains need too many passes (seeds +12 %).
-#ifndef IWPP_CHAINS
-#define IWPP_CHAINS 2
-#endif
-
-#ifndef IWPP_SCAN_VEC
-#define IWPP_SCAN_VEC 0   // 1: the scan kernels copy strips with 16-byte asynchronous copies where rows allow
-#endif
+constexpr int kCoopChains = 2;
 
 template <typename T, int CONN>
 __host__ __device__ constexpr size_t coop_smem_bytes() {
     return RegTile<T, CONN, kCoopStrip>::smem_per_warp(0) * kWarpsPerCta + sizeof(CoopShared);
 }
-// The scan kernels' staging area for 16-byte copies follows the drain's layout (16-byte aligned).
 template <typename T, int CONN>
-__host__ __device__ constexpr size_t coop_scan_stage_offset() {
-    return (coop_smem_bytes<T, CONN>() + 15) & ~(size_t)15;
-}
-template <typename T, int CONN>
-size_t coop_smem_fn(uint32_t) {
-    return IWPP_SCAN_VEC ? coop_scan_stage_offset<T, CONN>() + kWarpsPerCta * RegTile<T, CONN, kCoopStrip>::kStageBytes
-                         : coop_smem_bytes<T, CONN>();
-}
+size_t coop_smem_fn(uint32_t) { return coop_smem_bytes<T, CONN>(); }
 
 // Fold one strip's notification values (3 x 3 grid around the strip) into the CTA tile's:
 // the strip's top side is the tile's only for warp 0 (inside the tile otherwise, where the
@@ -132,7 +118,7 @@ __device__ void visit_tile_coop(const EngineArgs &a, const ImageView &im, uint32
         bool up_fresh = false;   // the strip's last pass was an up pass run with its current halo
         for (;;) {   // joint iterations of the strips
             if (!settled) {
-                const uint32_t sd = RT::template pass_chains<1, IWPP_CHAINS, HI>(J, I, jt, k16);
+                const uint32_t sd = RT::template pass_chains<1, kCoopChains, HI>(J, I, jt, k16);
                 const bool chd = sd != sum;   // (a round's first: the halo absorbed before it too)
                 sum = sd;
                 passes++;
@@ -142,7 +128,7 @@ __device__ void visit_tile_coop(const EngineArgs &a, const ImageView &im, uint32
                 if (up_fresh && !__any_sync(0xffffffffu, chd)) {
                     settled = true;
                 } else {
-                    const uint32_t su = RT::template pass_chains<-1, IWPP_CHAINS, HI>(J, I, jb, k16);
+                    const uint32_t su = RT::template pass_chains<-1, kCoopChains, HI>(J, I, jb, k16);
                     const bool chu = su != sum;
                     sum = su;
                     passes++;
@@ -291,13 +277,13 @@ __global__ void __launch_bounds__(kThreads, MIXED ? kRegBlocks
 // (a.tile_sweeps[t], else a.sweeps), the strips exchanging their boundary rows after each
 // pair, store what changed and notify the neighbours whose halo pixels the tile can now
 // raise; queue the tile if one of its pixels can still rise.
-template <typename T, int CONN, bool SWEEPS>
+template <typename T, int CONN>
 __device__ void scan_tile_coop(const EngineArgs &a, const ImageView &im, uint32_t t, uint8_t *wsmem,
-                               CoopShared &C, uint8_t *stage, int w, int lane) {
+                               CoopShared &C, int w, int lane) {
     constexpr int TH = kCoopStrip;
     using RT = RegTile<T, CONN, TH>;
-    const int sweeps = !SWEEPS ? 0 : a.tile_sweeps ? (int)a.tile_sweeps[t] : a.sweeps;   // CTA-uniform
-    if (SWEEPS && a.sweep_only && sweeps == 0) return;   // the sweeps-only pass: nothing to do here
+    const int sweeps = a.tile_sweeps ? (int)a.tile_sweeps[t] : a.sweeps;   // CTA-uniform
+    if (a.sweep_only && sweeps == 0) return;   // the sweeps-only pass: nothing to do here
     const long long c0 = clock64();
     const typename RT::Smem s = RT::carve(wsmem);
     const uint32_t *hx = RT::halo_words(s, lane);
@@ -305,13 +291,7 @@ __device__ void scan_tile_coop(const EngineArgs &a, const ImageView &im, uint32_
     const int ty = (int)(lt / im.tiles_x), tx = (int)(lt % im.tiles_x);
     const int y0 = ty * kCoopRows + TH * w, x0 = tx * RT::TW;
     uint32_t J[TH], I[TH], jt, jb, it, ib;
-#if IWPP_SCAN_VEC
-    if (RT::vec_ok(im, x0)) RT::load_vec(im, s, stage, y0, x0, J, I, jt, jb, it, ib, lane);
-    else RT::load(im, s, y0, x0, J, I, jt, jb, it, ib, lane);
-#else
-    (void)stage;
     RT::load(im, s, y0, x0, J, I, jt, jb, it, ib, lane);
-#endif
     bool bad = false;
 #pragma unroll
     for (int r = 0; r < TH; r++) bad |= max2(J[r], I[r]) != I[r];
@@ -359,9 +339,9 @@ __device__ void scan_tile_coop(const EngineArgs &a, const ImageView &im, uint32_
 // 16-row strip of a tile with its halo, checks the precondition and whether one of its
 // pixels can rise; a strip that can makes its tile PENDING (batches: a fire-and-forget OR)
 // or notifies it (single images: the first notification queues the tile, later ones find it
-// PENDING). Warps go from strip to strip independently, 7 CTAs per SM. The block scan
-// (iwpp_scan.cuh) replaces it wherever one connectivity is compiled in; the mixed-kind build
-// keeps it (its kinds switch per strip).
+// PENDING). Warps go from strip to strip independently, 7 CTAs per SM. Batches of both
+// connectivities take it (each strip switches on its image's kind); where one connectivity is
+// compiled in the block scan (iwpp_scan.cuh) replaces it.
 #ifndef IWPP_SCAN_STRIP_MINB
 #define IWPP_SCAN_STRIP_MINB 7   // CTAs per SM of the strip scan (72 registers, no spills)
 #endif
@@ -394,7 +374,7 @@ __device__ void scan_strip_coop(const EngineArgs &a, const ImageView &im, uint32
     __syncwarp();   // the warp's halo buffers are reloaded for its next strip
 }
 
-template <typename T, int CONN, bool MIXED>
+template <typename T, int CONN>
 __global__ void __launch_bounds__(kThreads, IWPP_SCAN_STRIP_MINB) scan_strip_coop_kernel(EngineArgs a) {
     using RT = RegTile<T, CONN, kCoopStrip>;
     extern __shared__ __align__(16) uint8_t smem_raw[];
@@ -405,10 +385,6 @@ __global__ void __launch_bounds__(kThreads, IWPP_SCAN_STRIP_MINB) scan_strip_coo
         const uint32_t t = (uint32_t)(u / kWarpsPerCta);
         const int sw = (int)(u % kWarpsPerCta);
         const ImageView &im = image_of(a, t);
-        if (!MIXED) {
-            scan_strip_coop<T, CONN>(a, im, t, sw, wsmem, lane);
-            continue;
-        }
         switch (im.kind) {
             case 0: scan_strip_coop<uint8_t, 4>(a, im, t, sw, wsmem, lane); break;
             case 1: scan_strip_coop<uint16_t, 4>(a, im, t, sw, wsmem, lane); break;
@@ -418,31 +394,29 @@ __global__ void __launch_bounds__(kThreads, IWPP_SCAN_STRIP_MINB) scan_strip_coo
     }
 }
 
-// The scan on whole tiles: SWEEPS, the build that runs sweep pairs (plans with sweeps,
-// per-tile sweep counts; the strips exchange boundary rows after each pair); the other one
-// is the lean scan with CTA barriers (the strip scan above replaces it).
-template <typename T, int CONN, bool MIXED, bool SWEEPS>
-__global__ void __launch_bounds__(kThreads, SWEEPS ? 4 : 8) scan_coop_kernel(EngineArgs a) {
+// The scan on whole tiles that runs sweep pairs (plans with sweeps, per-tile sweep counts); the
+// strips exchange boundary rows after each pair.
+template <typename T, int CONN, bool MIXED>
+__global__ void __launch_bounds__(kThreads, 4) scan_coop_kernel(EngineArgs a) {
     using RT = RegTile<T, CONN, kCoopStrip>;
     extern __shared__ __align__(16) uint8_t smem_raw[];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     uint8_t *wsmem = smem_raw + w * RT::smem_per_warp(0);
     CoopShared &C = *reinterpret_cast<CoopShared *>(smem_raw + kWarpsPerCta * RT::smem_per_warp(0));
-    uint8_t *stage = smem_raw + coop_scan_stage_offset<T, CONN>() + w * RT::kStageBytes;
     auto tile = [&](uint32_t t) {
         const ImageView &im = image_of(a, t);
         if (!MIXED) {
-            scan_tile_coop<T, CONN, SWEEPS>(a, im, t, wsmem, C, stage, w, lane);
+            scan_tile_coop<T, CONN>(a, im, t, wsmem, C, w, lane);
             return;
         }
         switch (im.kind) {
-            case 0: scan_tile_coop<uint8_t, 4, SWEEPS>(a, im, t, wsmem, C, stage, w, lane); break;
-            case 1: scan_tile_coop<uint16_t, 4, SWEEPS>(a, im, t, wsmem, C, stage, w, lane); break;
-            case 2: scan_tile_coop<uint8_t, 8, SWEEPS>(a, im, t, wsmem, C, stage, w, lane); break;
-            default: scan_tile_coop<uint16_t, 8, SWEEPS>(a, im, t, wsmem, C, stage, w, lane); break;
+            case 0: scan_tile_coop<uint8_t, 4>(a, im, t, wsmem, C, w, lane); break;
+            case 1: scan_tile_coop<uint16_t, 4>(a, im, t, wsmem, C, w, lane); break;
+            case 2: scan_tile_coop<uint8_t, 8>(a, im, t, wsmem, C, w, lane); break;
+            default: scan_tile_coop<uint16_t, 8>(a, im, t, wsmem, C, w, lane); break;
         }
     };
-    if (SWEEPS && a.sweep_only) {
+    if (a.sweep_only) {
         // The sweeps-only pass of learned batches, where most tiles have no sweeps: the CTA
         // reads the counts of kThreads of its tiles at once and visits only those with sweeps
         // (the same tiles as the loop below, grouped differently).

@@ -6,22 +6,18 @@
 
 namespace iwpp {
 
-#ifndef IWPP_SCAN_BLOCK
-#define IWPP_SCAN_BLOCK 1   // 0: the strip scan for every build (measured)
-#endif
-
 template <typename T, int CONN, bool MIXED = false>
 static RegKernelSet coop_set() {
     RegKernelSet k;
     // the block scan for builds of one connectivity; the mixed-kind build switches kinds
     // per strip in the strip scan
-    if constexpr (MIXED || !IWPP_SCAN_BLOCK) k.scan = scan_strip_coop_kernel<T, CONN, MIXED>;
+    if constexpr (MIXED) k.scan = scan_strip_coop_kernel<T, CONN>;
     else k.scan = scan_block_kernel<T, CONN, false>;
     k.drain = drain_coop_kernel<T, CONN, MIXED>;
     if constexpr (MIXED || std::is_same<T, AnyPix>::value) k.drain_hi = nullptr;   // batches: one build
     else k.drain_hi = drain_coop_kernel<T, CONN, MIXED, true>;
     k.smem = &coop_smem_fn<T, CONN>;
-    k.scan_sweeps = scan_coop_kernel<T, CONN, MIXED, true>;
+    k.scan_sweeps = scan_coop_kernel<T, CONN, MIXED>;
     // features in the scan: not for the mixed-kind build
     if constexpr (MIXED) k.scan_feats = nullptr;
     else k.scan_feats = scan_block_kernel<T, CONN, true>;
