@@ -34,8 +34,13 @@ constexpr int kCoopBlocks = IWPP_COOP_MINB;   // CTAs per SM of the cooperative 
 constexpr int kCoopBatchBlocks = IWPP_COOP_BATCH_MINB;
 // Its build for single dilations of at least kCoopHiTiles tiles (drain_hi). Measured, 6 CTAs per SM
 // -> this build: 4096 tiles h-dome 468 -> 467 us, 8836 tiles 718 -> 700 (seeds 1744 -> 1750), 16384
-// tiles 1248 -> 1204 (seeds 2173 -> 2115), 36864 tiles u16 2650 -> 2520, 65536 tiles seeds 9000 -> 8565;
-// erosions (fill-holes) are bound by tile hops up to the largest size and lose 3-5 %.
+// tiles 1248 -> 1204 (seeds 2173 -> 2115), 36864 tiles u16 2650 -> 2520, 65536 tiles seeds 9000 -> 8565.
+// Fill-holes markers (values travel from the border inwards) are bound by tile hops up to the
+// largest size and lose 3-5 % with it. The host cannot see the marker, and the operator stands in for
+// it: a dilation is taken for a dome or seeds, an erosion for fill-holes. An erosion and a
+// dilation do the same work, so a complemented image gets the other build: 16384 tiles border marker
+// 4490 us as an erosion, 4700 as a dilation; h-dome 1200 as a dilation, 1241 as an erosion;
+// seeds 2103 and 2159.
 constexpr int kCoopHiBlocks = 7;
 constexpr uint32_t kCoopHiTiles = 8192;
 RegKernelSet reg_kernel_set(int th, int tw, int v);

@@ -349,9 +349,9 @@ struct RegTile {
     // permutes issue every second cycle of a scheduler, shuffles every fourth (measured). DIR +1: down, halo =
     // the row above the tile; -1: up, halo = the row below. Returns the sum of the lane's pixels
     // (value_sum): values never fall, so a pass changed a pixel exactly when the sum is another. The sum
-    // is one dp2a per row, which issues beside the min / max / permute pipe that bounds a
-    // pass (measured), where an OR of the changed bits took that pipe's slots: 12 -> 10 of its
-    // cycles per row. MULADD: pair the neighbours by multiply-adds (k16).
+    // is one dp2a per row; with an OR of the changed bits instead the calls took longer (4096^2 4 %,
+    // 16384^2 seeds 4.7 %, 48 images 1.6 %, 256 learned 2.6 %; which unit that OR waits for was not
+    // measured). MULADD: pair the neighbours by multiply-adds (k16).
     template <int DIR, int NCH, bool MULADD>
     static __device__ __forceinline__ uint32_t pass_chains(uint32_t (&J)[TH], const uint32_t (&I)[TH], uint32_t halo,
                                                            uint32_t k16) {
