@@ -343,7 +343,7 @@ __device__ void scan_tile_coop(const EngineArgs &a, const ImageView &im, uint32_
 // connectivities take it (each strip switches on its image's kind); where one connectivity is
 // compiled in the block scan (iwpp_scan.cuh) replaces it.
 #ifndef IWPP_SCAN_STRIP_MINB
-#define IWPP_SCAN_STRIP_MINB 7   // CTAs per SM of the strip scan (72 registers, no spills)
+#define IWPP_SCAN_STRIP_MINB 7   // CTAs per SM of the strip scan (72 registers, 104 B of spills)
 #endif
 template <typename T, int CONN>
 __device__ void scan_strip_coop(const EngineArgs &a, const ImageView &im, uint32_t t, int sw, uint8_t *wsmem,

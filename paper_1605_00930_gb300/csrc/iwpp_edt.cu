@@ -11,10 +11,10 @@
 // Distances are squared Euclidean, exact in 32-bit integers for sides below 32768.
 //
 // Large images are bound by how many row steps are run and by how well their instructions are
-// fetched and overlapped, small ones (fewer tiles than the 4864 resident warps) and long chains of tiles by the
+// fetched and overlapped, small ones (fewer tiles than the 4864 warps of a full grid) and long chains of tiles by the
 // latency of a row step and of a visit's loads and stores. The tile lies in shared memory, not in
-// registers, so that the passes are loops over a row index: the code is a few hundred instructions
-// instead of 2 x 16 unrolled rows (whose fetches were the largest stall), 32 warps fit an SM
+// registers, so that the passes are loops over a row index: one row step per direction in the code
+// instead of 2 x 16 (whose fetches were the largest stall), 32 warps fit an SM
 // instead of 8, and rows without foreground, or whose neighbours have not changed, are skipped by
 // bit masks. For the latency, rows that follow one another are a run (edt_pass), a row step takes minima
 // of three (edt_step), and a visit's loads and stores go out together. The distances are written

@@ -29,7 +29,7 @@ constexpr int kRegBlocks = 4, kRegHiBlocks = 6;
 #endif
 constexpr int kCoopBlocks = IWPP_COOP_MINB;   // CTAs per SM of the cooperative solver's persistent kernel
 #ifndef IWPP_COOP_BATCH_MINB
-#define IWPP_COOP_BATCH_MINB 7   // its build for u8 + u16 batches (72 registers, 44 B of spills)
+#define IWPP_COOP_BATCH_MINB 7   // its build for u8 + u16 batches (72 registers, 24-32 B of spills)
 #endif
 constexpr int kCoopBatchBlocks = IWPP_COOP_BATCH_MINB;
 // Its build for single dilations of at least kCoopHiTiles tiles (drain_hi). Measured, 6 CTAs per SM

@@ -26,8 +26,8 @@
 
 namespace iwpp {
 
-// CTAs (of 4 warps) per SM: one pixel type 8 (64 registers; 12 and 6 are slower, 4096^2 u8 18.1 us
-// against 24.3 and 19.7), u8 + u16 6 (their variants spill at 64: 48 images 153 us against 161),
+// CTAs (of 4 warps) per SM: one pixel type 8 (64 registers, the u16 builds with
+// 220-300 B of spills; 12 and 6 are slower, 4096^2 u8 18.1 us against 24.3 and 19.7), u8 + u16 6 (their variants spill at 64: 48 images 153 us against 161),
 // with the feature sums 4 (256 images: 1.08 ms against 1.20 with 6 and 1.27 with 5).
 #ifndef IWPP_SCAN_MINB
 #define IWPP_SCAN_MINB 8

@@ -5,15 +5,16 @@
 // A row step of these operators weighs 60-100 instructions, so the drain is bound by how many
 // row steps it runs and by the warps there are to overlap them; small images by the chain of row
 // steps between two barriers. With the tile in shared memory the passes are loops over a row index:
-// the code stays a few hundred instructions, a thread needs 64-80 registers instead of 150-250, so
-// three times as many warps fit, and only the rows whose
-// neighbours changed are run, by three bit masks per strip: n, a pixel may change through
-// the row above; s, through the row below; h, through its own row. A down pass (rows top to
-// bottom) settles n, an up pass s, either h when it changes nothing. A tile that was visited
-// before starts with the rows next to its halo that the halo can change, and nothing else.
+// the code holds one row step per direction, a thread needs 64-80 registers instead of 150-250, so
+// three times as many warps fit, and only the rows whose neighbours changed are run, by three bit
+// masks per strip: n, a pixel may change through the row above; s, through the row below; h, through
+// its own row. A down pass (rows top to bottom) settles n, an up pass s, either h when it changes
+// nothing. A tile that was visited before starts with the rows next to its halo that the halo can
+// change, and nothing else.
 //
 // Strips exchange after one pass pair, eight strips of 8 rows. Both were chosen with rows that each
-// went through shared memory (and plain accesses between strips), calls with (warps, exchange):
+// went through shared memory (and plain accesses between strips), on inputs of their own, with
+// (warps, exchange):
 // watershed of 2048^2 u16 and 4096^2 u16, influence zones of 4096^2 and 1000^2:
 // (4, when clean) 1565 / 2742 / 1173 / 642 us, (4, pair) 1282 / 2489 / 1133 / 527, (8, when clean)
 // 1500 / 3119 / 1316 / 591, (8, pair) 1122 / 2946 / 1171 / 423, (8, single pass) 1432 / 2974 / 1217 / 458,
