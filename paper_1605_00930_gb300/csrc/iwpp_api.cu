@@ -2,9 +2,9 @@
 //
 // Host code only validates arguments, carves the caller's workspace and enqueues
 // kernels on the caller's stream:
-//   single image: workspace reset (memsets) -> tile-parallel scan kernel
+//   single image: workspace reset (one memset) -> tile-parallel scan kernel
 //     (precondition check, tile-local raster / anti-raster sweeps of Algorithm 7,
-//     frontier initialisation) -> persistent drain kernel (Algorithm 7's irregular
+//     frontier initialisation) -> queueing kernel -> persistent drain kernel (Algorithm 7's irregular
 //     propagation phase);
 //   batch: image-table upload (descriptors as kernel parameters) -> reset -> mixed
 //     scan kernel over every tile of every image (per-tile sweep counts) -> compact
